@@ -167,14 +167,14 @@ int lb_mass(lb_handle* h, double* mass);
 /* Wait for the stream and report latched device faults. */
 int lb_sync(lb_handle* h);
 
-/* Number of steps taken, and the launch shape in use: threads per block
- * (a multiple of 32; 10 of them are x-halo columns) and rows per segment. */
+/* Number of steps taken, and the launch shape in use: threads per block and
+ * rows per segment. */
 int lb_info(lb_handle* h, int64_t* steps, int* block_x, int* seg_rows, int* nblocks);
 
 /* Override the launch shape of the fused step (seg_rows >= 1; 0 keeps the
- * automatic choice; block_x 64, 128 or 256, 0 for the default: 64 up to
- * 4096 columns, 128 beyond). Results do not depend on the launch shape.
- * Used by the autotuner. */
+ * automatic choice; block_x 64, 128, 256 or 0: accepted, one block size
+ * serves them all). Results do not depend on the launch shape. Used by the
+ * autotuner. */
 int lb_set_launch(lb_handle* h, int block_x, int seg_rows);
 
 /* Checkpoint: lb_save_bytes gives the blob size; lb_save writes the state,
@@ -263,11 +263,12 @@ int lb_batch_init(lb_batch** b, const lb_batch_desc* d, int n, void* dev_workspa
  * instances for 32 steps. Runs of 32 steps are replayed from a captured
  * CUDA graph on a private stream ordered after and before `stream`.
  * Asynchronous. Results per instance are identical to stepping the instance
- * alone with the same block size. */
+ * alone. */
 int lb_batch_step(lb_batch* b, int nsteps);
 
-/* Launch shape shared by all instances: block_x 64 or 128; seg_rows 0 gives
- * every instance a share of one full wave proportional to its cells. */
+/* Launch shape shared by all instances: block_x 64 or 128 (one block size
+ * serves both); seg_rows 0 gives every instance a share of one full wave
+ * proportional to its cells. */
 int lb_batch_set_launch(lb_batch* b, int block_x, int seg_rows);
 
 /* Persistent mode (the batched boiling curve of Sec. 3.2-3.3 in one launch
@@ -276,12 +277,12 @@ int lb_batch_set_launch(lb_batch* b, int block_x, int seg_rows);
  * through runs of 32 steps, each run ONE cooperative launch of a fixed grid
  * (at most the blocks that fit on the GPU at once) replayed from a captured
  * CUDA graph, and the rest of the steps in one more launch. The instances
- * are cut into tiles (a block's two column strips x a segment of rows;
+ * are cut into tiles (a block's column strips x a segment of rows;
  * with seg_rows 0 the segments give about tiles_per_block tiles per block),
  * the tiles are dealt out to the blocks (longest first to the least loaded
  * block), and a tile starts a step once every tile of its instance has
  * finished the previous one. Results are bit-identical to stepping each
- * instance alone with the same block size. Each of those waits polls a
+ * instance alone. Each of those waits polls a
  * device counter at most wait_limit times (<= 0: the default, about 1-2
  * seconds); a wait that runs out ends its block and latches LB_E_TIMEOUT,
  * which lb_batch_sync and lb_batch_heat_flux report (the instances are then

@@ -11,12 +11,7 @@
 namespace lbgpu {
 
 constexpr int HALO = 5;    // x-halo columns per side recomputed by a block
-// the narrowest block (64 threads) covers 2 (64 - 2 HALO) = 108 columns, so a
-// grid has at most ceil(Lx / 108) strips: the heat-flux slots per instance
-constexpr int MIN_STRIP_COLS = 2 * (64 - 2 * HALO);
-constexpr int RING = 4;    // rows kept per stencil field in shared memory
-constexpr int TRING = 8;   // rows kept of theta^t
-constexpr int SM_ROWS = 7 * RING + TRING;  // psi rho vx vy u2 u3 u4 + theta
+constexpr int TILE_COLS = 54;    // columns of a strip (64 less the halos); a block owns two
 
 enum { BC_WALLS = 0, BC_TOP_OUTFLOW = 1, BC_PERIODIC = 2 };
 enum : unsigned { ERR_EOS = 1u, ERR_NONFINITE = 2u, ERR_BOUNDS = 4u, ERR_TIMEOUT = 8u };
@@ -40,12 +35,14 @@ struct StepParams {
     float* th_out;
     const float* thb;   // theta_b(x) = T_b(x) - T_s on the bottom wall
     Acc* acc;
-    // one slot per column strip of the bottom segment: the strip's sum of
-    // q_w for the step in flight, folded in strip order by the last strip
+    // the columns' terms of q(t) (fold_heat, lb_common.cuh): written by this step,
+    // and those of the step before
     double* qpart;
+    const double* qprev;
+    double qscale;  // -c_v chi / (2 Lx)
     int Lx, Ly, pitch, plane;
     int bc, ghost, isothermal;
-    int nout, nstrips, seg_h;
+    int nstrips, seg_h;
     // Peng-Robinson EOS (Eq. 21): phi(T) = (k0 - k1 sqrt(T))^2 with
     // k0 = 1 + kappa, k1 = kappa / sqrt(Tc); psi^2 = two_over_G (p - rho/3).
     float Ts, a, b, R, two_over_G, k0, k1, G;
@@ -115,6 +112,16 @@ __device__ __forceinline__ float lb_ldg(const float* p, const float*, size_t, Ac
 __device__ __forceinline__ float lb_ldco(const float* p, const float*, size_t, Acc*) { return *p; }
 __device__ __forceinline__ void lb_st(float* p, float v, const float*, size_t, Acc*) { *p = v; }
 #endif
+// A store that only lanes with `on` make, as one predicated instruction: a
+// branch around a group of stores would end the basic block and with it the
+// compiler's freedom to interleave two rows' arithmetic.
+__device__ __forceinline__ void lb_st_if(bool on, float* p, float v, const float* base, size_t n, Acc* acc) {
+#ifdef LB_CHECKED
+    if (on) lb_st(p, v, base, n, acc);
+#else
+    asm volatile("{ .reg .pred q; setp.ne.u32 q, %2, 0; @q st.global.f32 [%0], %1; }" ::"l"(p), "f"(v), "r"((unsigned)on));
+#endif
+}
 // Loads of the step's input state: through the read-only path in a kernel
 // that runs one step (lb_ldg), as plain coherent loads (lb_ldco) in the
 // persistent batch, where other blocks rewrite the buffers during the launch:

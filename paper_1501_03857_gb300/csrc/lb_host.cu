@@ -171,9 +171,8 @@ struct Layout {
     size_t plane, f0, f1, t0, t1, thb, acc, qpart, total;
 };
 
-// FP64 slots of the per-strip heat-flux sums (the most strips any launch
-// shape gives this width)
-inline size_t qpart_bytes(int Lx) { return sizeof(double) * (size_t)((Lx + MIN_STRIP_COLS - 1) / MIN_STRIP_COLS); }
+// FP64 terms of q(t), one per column, of the step in flight and the one before
+inline size_t qpart_bytes(int Lx) { return 2 * sizeof(double) * (size_t)Lx; }
 
 Layout layout(const lb_grid* g) {
     Layout L;
@@ -254,7 +253,6 @@ void fill_params(lb_handle* h) {
     const lb_thermal& t = h->th;
     P.thb = h->thb;
     P.acc = h->acc;
-    P.qpart = h->qpart;
     P.Lx = g.Lx;
     P.Ly = g.Ly;
     P.pitch = h->lay.pitch;
@@ -289,42 +287,48 @@ void fill_params(lb_handle* h) {
     P.chi = (float)(t.cv_chi / t.cv);
     P.cvchi = (float)t.cv_chi;
     P.inv_cv = (float)(1.0 / t.cv);
+    P.qscale = -0.5 * (double)P.cvchi / (double)g.Lx;
     set_pairs(P);
 }
 
-// The launch shape of the fused step for this grid (block_x, seg_rows 0:
-// automatic).
+// The parameters of a step from buffer `cur`.
+StepParams step_params(const lb_handle* h, const StepParams& base, int cur) {
+    StepParams P = base;
+    P.f_in = h->f[cur];
+    P.f_out = h->f[1 - cur];
+    P.th_in = h->t[cur];
+    P.th_out = h->t[1 - cur];
+    P.qpart = h->qpart + (size_t)cur * P.Lx;
+    P.qprev = h->qpart + (size_t)(1 - cur) * P.Lx;
+    return P;
+}
+
+inline int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
+
+// Column strips of a step's blocks.
+inline int form_strips(int form, int Lx) {
+    (void)form;
+    return ceil_div(Lx, 2 * TILE_COLS);
+}
+
+// The launch shape of the fused step for this grid (seg_rows 0: segments that
+// fill the GPU once).
 int compute_launch(const lb_handle* h, int block_x, int seg_rows, Launch* out) {
-    int dev = 0, nsm = 0;
+    int dev = 0, nsm = 0, occ = 0, threads = 0;
     LB_CUDA(cudaGetDevice(&dev), "cudaGetDevice");
     LB_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev), "cudaDeviceGetAttribute");
-    const int Lx = h->grid.Lx, Ly = h->grid.Ly;
-    // 64 threads up to 4096 columns, 128 beyond (measured: 64 is 1-5 %
-    // faster on 1024^2-4096^2, 128 2 % faster on 8192^2)
-    int bx = block_x, occ = 0;
-    if (bx <= 0) bx = Lx <= 4096 ? 64 : 128;
-    if (!dual_supported(bx)) return fail(LB_E_INVAL, "the fused step takes block_x 64, 128 or 256, not %d", bx);
-    LB_CUDA(dual_occupancy(bx, &occ), "occupancy");
-    if (occ < 1) return fail(LB_E_INVAL, "block_x %d does not fit on an SM", bx);
-    const int nout = bx - 2 * HALO;
-    const int cols = 2 * nout;  // output columns per block
-    const int nstrips = (Lx + cols - 1) / cols;
-    int seg = seg_rows;
-    if (seg <= 0) {
-        const int slots = nsm * occ;
-        const int nseg = std::max(1, slots / nstrips);
-        seg = std::max(8, (Ly + nseg - 1) / nseg);
-    }
-    out->block_x = bx;
-    out->seg_rows = seg;
-    out->nstrips = nstrips;
-    out->nseg = (Ly + seg - 1) / seg;
+    if (block_x != 0 && block_x != 64 && block_x != 128 && block_x != 256)
+        return fail(LB_E_INVAL, "the fused step takes block_x 64, 128 or 256, not %d", block_x);
+    LB_CUDA(step_occupancy(FORM_MARCH, &threads, &occ), "occupancy");
+    if (occ < 1) return fail(LB_E_INVAL, "the fused step's block of %d threads does not fit on an SM", threads);
+    const int nstrips = form_strips(FORM_MARCH, h->grid.Lx);
+    const int seg = seg_rows > 0 ? seg_rows : std::max(8, ceil_div(h->grid.Ly, std::max(1, nsm * occ / nstrips)));
+    *out = Launch{FORM_MARCH, threads, seg, nstrips, ceil_div(h->grid.Ly, seg)};
     return LB_OK;
 }
 
 // The step parameters that describe launch shape L.
 void apply_launch(StepParams& P, const Launch& L) {
-    P.nout = L.block_x - 2 * HALO;
     P.nstrips = L.nstrips;
     P.seg_h = L.seg_rows;
 }
@@ -411,13 +415,11 @@ int aux_stream(lb_handle* h) {
     return LB_OK;
 }
 
-int launch_one(lb_handle* h, const StepParams& base, int cur, cudaStream_t q) {
-    StepParams P = base;
-    P.f_in = h->f[cur];
-    P.f_out = h->f[1 - cur];
-    P.th_in = h->t[cur];
-    P.th_out = h->t[1 - cur];
-    LB_CUDA(launch_step(P, h->launch, q), "step launch");
+// One step from buffer `cur`; fold: the step before it belongs to the same
+// call (launch_step).
+int launch_one(lb_handle* h, const StepParams& base, int cur, bool fold, cudaStream_t q) {
+    const StepParams P = step_params(h, base, cur);
+    LB_CUDA(launch_step(P, h->launch, fold, q), "step launch");
     if (h->probe.n > 0) {
         ProbeArgs A = h->probe;
         A.f = P.f_out;
@@ -427,16 +429,18 @@ int launch_one(lb_handle* h, const StepParams& base, int cur, cudaStream_t q) {
     return LB_OK;
 }
 
+// q(t) of the last step, which left buffer `cur`, into the statistics.
+int fold_last(lb_handle* h, const StepParams& base, int cur, cudaStream_t q) {
+    if (base.bc != BC_PERIODIC) LB_CUDA(launch_fold(step_params(h, base, cur), q), "heat flux launch");
+    return LB_OK;
+}
+
 int run_steps(lb_handle* h, const StepParams& base, int nsteps) {
     int left = nsteps;
     if (left >= STEP_GRAPH) {
         int rc = aux_stream(h);
         if (rc) return rc;
-        StepParams first = base;
-        first.f_in = h->f[h->cur];
-        first.f_out = h->f[1 - h->cur];
-        first.th_in = h->t[h->cur];
-        first.th_out = h->t[1 - h->cur];
+        const StepParams first = step_params(h, base, h->cur);
         cudaGraphExec_t exec = nullptr;
         for (auto& g : h->step_graphs)
             if (memcmp(&g.first, &first, sizeof(StepParams)) == 0 && memcmp(&g.launch, &h->launch, sizeof(Launch)) == 0 &&
@@ -446,7 +450,8 @@ int run_steps(lb_handle* h, const StepParams& base, int nsteps) {
         if (!exec) {
             cudaGraph_t graph = nullptr;
             LB_CUDA(cudaStreamBeginCapture(gs, cudaStreamCaptureModeThreadLocal), "begin capture");
-            for (int k = 0; k < STEP_GRAPH && rc == LB_OK; ++k) rc = launch_one(h, base, h->cur ^ (k & 1), gs);
+            for (int k = 0; k < STEP_GRAPH && rc == LB_OK; ++k) rc = launch_one(h, base, h->cur ^ (k & 1), k > 0, gs);
+            if (rc == LB_OK) rc = fold_last(h, base, h->cur, gs);
             cudaError_t e = cudaStreamEndCapture(gs, &graph);
             if (rc) {
                 if (graph) cudaGraphDestroy(graph);
@@ -471,13 +476,14 @@ int run_steps(lb_handle* h, const StepParams& base, int nsteps) {
         LB_CUDA(cudaEventRecord(h->adj_out, gs), "cudaEventRecord");
         LB_CUDA(cudaStreamWaitEvent(h->st, h->adj_out, 0), "cudaStreamWaitEvent");
     }
-    for (; left > 0; --left) {
-        int rc = launch_one(h, base, h->cur, h->st);
+    const bool some = left > 0;
+    for (bool fold = false; left > 0; --left, fold = true) {
+        int rc = launch_one(h, base, h->cur, fold, h->st);
         if (rc) return rc;
         h->cur ^= 1;
         h->steps++;
     }
-    return LB_OK;
+    return some ? fold_last(h, base, h->cur, h->st) : LB_OK;
 }
 
 }  // namespace
@@ -591,7 +597,8 @@ int lb_init(lb_handle** out, const lb_grid* grid, const lb_eos* eos, const lb_th
     }
     h->rho_ave = sum / ((double)Lx * Ly);
     fill_params(h);
-    cudaError_t e = dual_prepare();
+    cudaError_t e = step_prepare();
+    if (e == cudaSuccess) e = recompute_prepare();
     if (e != cudaSuccess) { release(h); return cuda_fail(e, "cudaFuncSetAttribute"); }
     rc = choose_launch(h, 0, 0);
     if (rc) { release(h); return rc; }
@@ -924,7 +931,8 @@ struct lb_batch {
     int* block_off;              // device [n + 1]: first block of each instance
     std::vector<int> h_off;
     std::vector<StepParams> h_table;
-    int block_x, seg_req;        // launch shape (seg_req 0: automatic)
+    int block_x, seg_req;        // launch shape asked for (seg_req 0: automatic)
+    int form, threads;           // the form in use and its block size
     int nblocks;
     bool dirty;                  // tables no longer match the instances' buffers
     int64_t steps;
@@ -964,12 +972,11 @@ size_t batch_tail_offset(const lb_batch_desc* d, int n, std::vector<size_t>* off
     return off;
 }
 
-// Most tiles a batch can have: the 64-thread blocks' strips (the narrowest)
-// and segments of one row.
+// Most tiles a batch can have: the narrowest strips and segments of one row.
 long long batch_max_tiles(const lb_batch_desc* d, int n) {
     long long t = 0;
     for (int i = 0; i < n; ++i)
-        t += (long long)((d[i].grid.Lx + MIN_STRIP_COLS - 1) / MIN_STRIP_COLS) * d[i].grid.Ly;
+        t += (long long)form_strips(FORM_MARCH, d[i].grid.Lx) * d[i].grid.Ly;
     return t;
 }
 
@@ -1009,60 +1016,55 @@ void batch_constants(lb_batch* b) {
         if (!same_constants(h->base, b->kconst)) b->kshared = false;
 }
 
-// Common block size, per-instance segment height and block offsets. With an
-// automatic segment height every instance gets a share of one full wave
-// proportional to its cells (tpb waves' worth in the persistent mode, whose
-// grid is one wave that takes about tpb tiles per block).
-int batch_layout(lb_batch* b) {
-    const int n = (int)b->inst.size();
-    int dev = 0, nsm = 0, occ = 0;
-    LB_CUDA(cudaGetDevice(&dev), "cudaGetDevice");
-    LB_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev), "cudaDeviceGetAttribute");
-    batch_constants(b);
-    if (b->tpb > 0) LB_CUDA(persist_occupancy(b->block_x, b->kshared, &occ), "occupancy");
-    else LB_CUDA(batch_occupancy(b->block_x, b->kshared, &occ), "occupancy");
-    if (occ < 1) return fail(LB_E_INVAL, "batch block_x %d does not fit on an SM", b->block_x);
-    const int waves = std::max(1, b->tpb);
-    const int nout = b->block_x - 2 * HALO;
-    // Without a requested height every tile gets about the same number of
-    // rows: a block costs its rows (plus the pipeline's halo) whatever share
-    // of its columns the instance fills, and the step lasts as long as its
-    // longest tile. S is the smallest height at which the tiles still fit in
-    // `waves` waves; an instance splits its rows into ceil(Ly / S) equal
-    // segments.
-    auto nstrips_of = [&](const lb_handle* h) { return (h->grid.Lx + 2 * nout - 1) / (2 * nout); };
-    int S = 8;
-    if (b->seg_req <= 0) {
-        const long long cap = (long long)nsm * occ * waves;
-        auto tiles_at = [&](int height) {
-            long long t = 0;
-            for (lb_handle* h : b->inst) t += (long long)nstrips_of(h) * ((h->grid.Ly + height - 1) / height);
-            return t;
-        };
+// Rows per tile in a batch whose tiles fit in `cap` slots, and how many tiles
+// that makes. Without a
+// requested height every tile gets about the same number of rows: a block
+// costs its rows (plus the pipeline's halo) whatever share of its columns the
+// instance fills, and the step lasts as long as its longest tile.
+int batch_height(const lb_batch* b, int form, long long cap, long long* tiles) {
+    auto tiles_at = [&](int height) {
+        long long t = 0;
+        for (lb_handle* h : b->inst) t += (long long)form_strips(form, h->grid.Lx) * ceil_div(h->grid.Ly, height);
+        return t;
+    };
+    int S = b->seg_req;
+    if (S <= 0) {
         int hi = 8;
         for (lb_handle* h : b->inst) hi = std::max(hi, h->grid.Ly);
+        S = 8;
         while (S < hi) {  // the smallest height whose tiles fit (tiles_at falls as the height grows)
             const int mid = S + (hi - S) / 2;
             if (tiles_at(mid) <= cap) hi = mid;
             else S = mid + 1;
         }
     }
+    *tiles = tiles_at(S);
+    return S;
+}
+
+// Per-instance segment height and block offsets. With an automatic
+// segment height the tiles of all instances are about equal and fill one wave
+// (tpb waves in the persistent mode, whose grid is one wave that takes about
+// tpb tiles per block).
+int batch_layout(lb_batch* b) {
+    const int n = (int)b->inst.size();
+    int dev = 0, nsm = 0, occ = 0, S = 0;
+    LB_CUDA(cudaGetDevice(&dev), "cudaGetDevice");
+    LB_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev), "cudaDeviceGetAttribute");
+    batch_constants(b);
+    const int waves = std::max(1, b->tpb);
+    b->form = FORM_MARCH;
+    LB_CUDA(batch_occupancy(b->form, b->kshared, b->tpb > 0, &b->threads, &occ), "occupancy");
+    if (occ < 1) return fail(LB_E_INVAL, "the batched step's block of %d threads does not fit on an SM", b->threads);
+    long long tiles = 0;
+    S = batch_height(b, b->form, (long long)nsm * occ * waves, &tiles);
     b->h_off.assign(n + 1, 0);
     for (int i = 0; i < n; ++i) {
         lb_handle* h = b->inst[i];
-        const int nstrips = nstrips_of(h);
-        int seg = b->seg_req;
-        if (seg <= 0) {
-            const int nseg = (h->grid.Ly + S - 1) / S;
-            seg = (h->grid.Ly + nseg - 1) / nseg;
-        }
-        h->launch.block_x = b->block_x;
-        h->launch.seg_rows = seg;
-        h->launch.nstrips = nstrips;
-        h->launch.nseg = (h->grid.Ly + seg - 1) / seg;
-        h->base.nout = nout;
-        h->base.nstrips = nstrips;
-        h->base.seg_h = seg;
+        const int nstrips = form_strips(b->form, h->grid.Lx);
+        const int seg = b->seg_req > 0 ? b->seg_req : ceil_div(h->grid.Ly, ceil_div(h->grid.Ly, S));
+        h->launch = Launch{b->form, b->threads, seg, nstrips, ceil_div(h->grid.Ly, seg)};
+        apply_launch(h->base, h->launch);
         b->h_off[i + 1] = b->h_off[i] + nstrips * h->launch.nseg;
     }
     b->nblocks = b->h_off[n];
@@ -1149,13 +1151,7 @@ int batch_upload(lb_batch* b) {
     for (int p = 0; p < 2; ++p)
         for (int i = 0; i < n; ++i) {
             lb_handle* h = b->inst[i];
-            StepParams P = h->base;
-            const int c = h->cur ^ p;
-            P.f_in = h->f[c];
-            P.f_out = h->f[1 - c];
-            P.th_in = h->t[c];
-            P.th_out = h->t[1 - c];
-            b->h_table[p * n + i] = P;
+            b->h_table[p * n + i] = step_params(h, h->base, h->cur ^ p);
         }
     LB_CUDA(cudaMemcpyAsync(b->table, b->h_table.data(), 2 * n * sizeof(StepParams), cudaMemcpyHostToDevice, b->st),
             "batch table upload");
@@ -1163,11 +1159,18 @@ int batch_upload(lb_batch* b) {
     return LB_OK;
 }
 
-int batch_launch_one(lb_batch* b, cudaStream_t s, int parity) {
+int batch_launch_one(lb_batch* b, cudaStream_t s, int parity, bool fold) {
     const int n = (int)b->inst.size();
-    LB_CUDA(batch_launch(b->block_x, b->table + parity * n, b->block_off, n, b->nblocks,
-                         b->kshared ? &b->kconst : nullptr, s),
+    LB_CUDA(batch_launch(b->form, b->table + parity * n, b->block_off, n, b->nblocks,
+                         b->kshared ? &b->kconst : nullptr, fold, s),
             "batch step launch");
+    return LB_OK;
+}
+
+// q(t) of every instance's last step; parity: the table of the step to come.
+int batch_fold_last(lb_batch* b, cudaStream_t s, int parity) {
+    const int n = (int)b->inst.size();
+    LB_CUDA(batch_fold(b->table + parity * n, n, s), "batch heat flux launch");
     return LB_OK;
 }
 
@@ -1184,8 +1187,8 @@ int persist_launch_one(lb_batch* b, cudaStream_t s, int nsteps) {
     A.nsteps = nsteps;
     A.wait_limit = b->wait_limit;
     LB_CUDA(cudaMemsetAsync(b->d_arrive, 0, n * sizeof(unsigned), s), "clear arrival counters");
-    LB_CUDA(persist_launch(b->block_x, b->kshared ? &b->kconst : nullptr, A, b->pgrid, s), "persistent batch launch");
-    return LB_OK;
+    LB_CUDA(persist_launch(b->form, b->kshared ? &b->kconst : nullptr, A, b->pgrid, s), "persistent batch launch");
+    return batch_fold_last(b, s, nsteps & 1);
 }
 
 int persist_graph(lb_batch* b, cudaGraphExec_t* out) {
@@ -1212,7 +1215,8 @@ int batch_graph(lb_batch* b, cudaGraphExec_t* out) {
         cudaGraph_t g = nullptr;
         LB_CUDA(cudaStreamBeginCapture(b->gs, cudaStreamCaptureModeThreadLocal), "begin capture");
         int rc = LB_OK;
-        for (int k = 0; k < GRAPH_STEPS && rc == LB_OK; ++k) rc = batch_launch_one(b, b->gs, k & 1);
+        for (int k = 0; k < GRAPH_STEPS && rc == LB_OK; ++k) rc = batch_launch_one(b, b->gs, k & 1, k > 0);
+        if (rc == LB_OK) rc = batch_fold_last(b, b->gs, 0);
         cudaError_t e = cudaStreamEndCapture(b->gs, &g);
         if (rc) {
             if (g) cudaGraphDestroy(g);
@@ -1323,7 +1327,7 @@ int lb_batch_init(lb_batch** out, const lb_batch_desc* d, int n, void* dev_works
 
 int lb_batch_set_launch(lb_batch* b, int block_x, int seg_rows) {
     if (!b) return fail(LB_E_INVAL, "null batch");
-    if (!batch_supported(block_x)) return fail(LB_E_INVAL, "batch block_x must be 64 or 128, not %d", block_x);
+    if (block_x != 64 && block_x != 128) return fail(LB_E_INVAL, "batch block_x must be 64 or 128, not %d", block_x);
     if (seg_rows < 0) return fail(LB_E_INVAL, "seg_rows must be >= 0");
     b->block_x = block_x;
     b->seg_req = seg_rows;
@@ -1372,10 +1376,12 @@ int lb_batch_step(lb_batch* b, int nsteps) {
         LB_CUDA(cudaEventRecord(b->ev_out, b->gs), "cudaEventRecord");
         LB_CUDA(cudaStreamWaitEvent(b->st, b->ev_out, 0), "cudaStreamWaitEvent");
     }
-    for (; left > 0; --left, parity ^= 1) {
-        rc = batch_launch_one(b, b->st, parity);
+    const bool some = left > 0;
+    for (bool fold = false; left > 0; --left, parity ^= 1, fold = true) {
+        rc = batch_launch_one(b, b->st, parity, fold);
         if (rc) return rc;
     }
+    if (some && (rc = batch_fold_last(b, b->st, parity))) return rc;
     for (lb_handle* h : b->inst) {
         h->cur ^= (nsteps & 1);
         h->steps += nsteps;
@@ -1433,7 +1439,7 @@ int lb_batch_set_wettability(lb_batch* b, int i, double Gw) {
 int lb_batch_info(lb_batch* b, int64_t* steps, int* block_x, int* nblocks) {
     if (!b) return fail(LB_E_INVAL, "null batch");
     if (steps) *steps = b->steps;
-    if (block_x) *block_x = b->block_x;
+    if (block_x) *block_x = b->threads;
     if (nblocks) *nblocks = b->tpb > 0 ? b->pgrid : b->nblocks;
     return LB_OK;
 }
@@ -1579,19 +1585,24 @@ int lb_adjoint(lb_handle* h, int nsteps, int ckpt_every, void* dev_scratch, size
         // into checkpoint n+1 and the step's intermediates into set n, so the
         // reverse sweep replays nothing
         for (int n = 0; n < nsteps; ++n) {
-            StepParams P = base;
+            StepParams P = step_params(h, base, n & 1);
             P.acc = acc;
             P.f_in = sf(L.ckpt, n);
             P.th_in = sf(L.ckpt, n) + 9 * pl;
             P.f_out = sf(L.ckpt, n + 1);
             P.th_out = sf(L.ckpt, n + 1) + 9 * pl;
-            LB_CUDA(dual_recompute(P, rec_at(n), true, true, h->launch, st), "adjoint forward step");
+            LB_CUDA(launch_recompute(P, rec_at(n), true, true, n > 0, h->launch, st), "adjoint forward step");
             if (h->probe.n > 0) {
                 ProbeArgs A = h->probe;
                 A.f = P.f_out;
                 A.th = P.th_in;
                 LB_CUDA(launch_probe(A, st), "probe launch");
             }
+        }
+        {
+            StepParams P = base;
+            P.acc = acc;
+            if ((rc = fold_last(h, P, nsteps & 1, st))) return rc;
         }
         // the simulation advances as with the plain steps: the last state
         // into the current population and theta buffers (separate arrays of
@@ -1656,7 +1667,7 @@ int lb_adjoint(lb_handle* h, int nsteps, int ckpt_every, void* dev_scratch, size
             const bool out = j + 1 < len;
             P.f_out = out ? seg_state(buf, j + 1) : nullptr;
             P.th_out = out ? seg_state(buf, j + 1) + 9 * pl : nullptr;
-            LB_CUDA(dual_recompute(P, seg_rec(buf, j), out, false, h->launch, q), "adjoint recompute step");
+            LB_CUDA(launch_recompute(P, seg_rec(buf, j), out, false, false, h->launch, q), "adjoint recompute step");
         }
         return LB_OK;
     };

@@ -8,48 +8,53 @@
 
 namespace lbgpu {
 
-// Launch shape of the fused step (lb_step3.cu): block_x threads per block,
-// each thread owning one column of two strips of block_x - 2*HALO output
-// columns; seg_rows rows per block; nstrips x nseg blocks.
+// Forms of the fused step (lb_march.cuh).
+enum Form { FORM_MARCH = 0, FORM_COUNT = 1 };
+
+// Launch shape of the fused step: nstrips x nseg blocks of seg_rows rows
+// each; block_x threads per block (the form's).
 struct Launch {
-    int block_x, seg_rows, nstrips, nseg;
+    int form, block_x, seg_rows, nstrips, nseg;
 };
 
-// One step of the fused kernel: one row per iteration, two column strips per
-// block in paired FP32 (block_x 64, 128 or 256).
-bool dual_supported(int block_x);
-cudaError_t dual_prepare();  // opt in to the dynamic shared memory
-cudaError_t dual_occupancy(int block_x, int* blocks_per_sm);
-cudaError_t launch_step(const StepParams& P, const Launch& L, cudaStream_t st);
+cudaError_t step_prepare();  // opt in to the dynamic shared memory
+cudaError_t step_occupancy(int form, int* threads, int* blocks_per_sm);
+// One step. It leaves the columns' terms of q(t) in P.qpart; with fold it
+// adds the previous step's (P.qprev) to the heat-flux statistics, and after
+// the last step of a call launch_fold, given the parameters the next step
+// would have, adds the last one's.
+cudaError_t launch_step(const StepParams& P, const Launch& L, bool fold, cudaStream_t st);
+cudaError_t launch_fold(const StepParams& P, cudaStream_t st);
 
 // The forward intermediates of one step that the adjoint's reverse kernels
-// read (lb_adjoint.cu), written by the dual-strip step in its recompute mode
-// (lb_step3.cu) into pitched [Ly][pitch] planes. The gradients drx, dry and
+// read (lb_adjoint.cu), written by the fused step in its recompute mode
+// (lb_step_rec.cu) into pitched [Ly][pitch] planes. The gradients drx, dry and
 // div v carry the stencil weights; ax, ay are coefficients of K(T), Eq. 18
 // (0 on the wall rows; cA, cB and F_m follow from div v, rho and psi); u2-u4
 // the RK stage inputs (theta on the wall rows). With out the step itself is written too (f*, theta of the
 // next level to P.f_out, P.th_out), and with heat (only with out) q(t) is
-// added to P.acc's heat-flux sums as the plain step does.
+// accounted for as the plain step does (fold as there).
 struct RecomputeOut {
     float *rho, *psi;
     float *drx, *dry, *divv, *ax, *ay, *u2, *u3, *u4;
 };
 constexpr int kRecomputePlanes = 10;  // the planes of RecomputeOut, in its order
-cudaError_t dual_recompute(const StepParams& P, const RecomputeOut& R, bool out, bool heat, const Launch& L,
-                           cudaStream_t st);
+cudaError_t recompute_prepare();
+cudaError_t launch_recompute(const StepParams& P, const RecomputeOut& R, bool out, bool heat, bool fold,
+                             const Launch& L, cudaStream_t st);
 
-// The same step over a table of independent instances in one launch
-// (paired FP32, block_x 64 or 128); instance i owns blocks
+// The same step over a table of independent instances in one launch ; instance i owns blocks
 // [block_off[i], block_off[i+1]).
-bool batch_supported(int block_x);
 cudaError_t batch_prepare();
-cudaError_t batch_occupancy(int block_x, bool shared_k, int* blocks_per_sm);
-// K non-null: every instance shares the model constants in *K (see
-// step_body in lb_step3.cu) and the kernel reads them from its parameters.
-cudaError_t batch_launch(int block_x, const StepParams* table, const int* block_off, int n, int nblocks,
-                         const StepParams* K, cudaStream_t st);
+cudaError_t batch_occupancy(int form, bool shared_k, bool persistent, int* threads, int* blocks_per_sm);
+// K non-null: every instance shares the model constants in *K and the kernel
+// reads them from its parameters. fold as in launch_step, batch_fold as
+// launch_fold (given the table of the step that would follow).
+cudaError_t batch_launch(int form, const StepParams* table, const int* block_off, int n, int nblocks,
+                         const StepParams* K, bool fold, cudaStream_t st);
+cudaError_t batch_fold(const StepParams* table, int n, cudaStream_t st);
 
-// The persistent batch (lb_batch_persist in lb_step3.cu): one cooperative
+// The persistent batch (lb_batch_persist in lb_step_batch.cu): one cooperative
 // launch of a fixed grid advances every instance by nsteps steps; block g
 // takes tiles tile_off[g] .. tile_off[g+1]-1 (instance, block index within
 // the instance) every step, after all tiles of the instance finished the
@@ -66,8 +71,7 @@ struct PersistArgs {
     int n, nsteps;
     unsigned long long wait_limit;
 };
-cudaError_t persist_occupancy(int block_x, bool shared_k, int* blocks_per_sm);
-cudaError_t persist_launch(int block_x, const StepParams* K, const PersistArgs& A, int nblocks, cudaStream_t st);
+cudaError_t persist_launch(int form, const StepParams* K, const PersistArgs& A, int nblocks, cudaStream_t st);
 
 // Initial state: f* = w_a rho0 (rest equilibrium), theta = 0 with the wall
 // rows at their Dirichlet values. rho0 is pitched [Ly][pitch].
@@ -89,7 +93,7 @@ cudaError_t adjoint_grads_reset(const StepParams& P, void* work, cudaStream_t st
 // the wall rows and the outflow top, whose share is already in lf). Zero lf
 // and lr are a zero adjoint. The in and out planes are distinct buffers.
 // R holds the forward intermediates of the step being reversed (written by
-// dual_recompute from the same state).
+// launch_recompute from the same state).
 cudaError_t adjoint_reverse_step(const StepParams& P, const RecomputeOut& R, void* work, const float* fstar,
                                  const float* theta, const float* lf_in, const float* lt_in, const float* lr_in,
                                  float* lf_out, float* lt_out, float* lr_out, float lq, cudaStream_t st);
