@@ -171,10 +171,11 @@ int lb_sync(lb_handle* h);
  * rows per segment. */
 int lb_info(lb_handle* h, int64_t* steps, int* block_x, int* seg_rows, int* nblocks);
 
-/* Override the launch shape of the fused step (seg_rows >= 1; 0 keeps the
- * automatic choice; block_x 64, 128, 256 or 0: accepted, one block size
- * serves them all). Results do not depend on the launch shape. Used by the
- * autotuner. */
+/* Override the launch shape of the fused step: block_x names its form (64:
+ * blocks marching up column strips, for domains that fill the GPU; 128 and
+ * 256: tiles of 24 and 16 computed rows, for smaller ones; 0: the one
+ * expected to be fastest), seg_rows >= 1 the rows per block (0: automatic).
+ * Results do not depend on the launch shape. Used by the autotuner. */
 int lb_set_launch(lb_handle* h, int block_x, int seg_rows);
 
 /* Checkpoint: lb_save_bytes gives the blob size; lb_save writes the state,
@@ -266,9 +267,10 @@ int lb_batch_init(lb_batch** b, const lb_batch_desc* d, int n, void* dev_workspa
  * alone. */
 int lb_batch_step(lb_batch* b, int nsteps);
 
-/* Launch shape shared by all instances: block_x 64 or 128 (one block size
- * serves both); seg_rows 0 gives every instance a share of one full wave
- * proportional to its cells. */
+/* Launch shape shared by all instances: block_x 64 (the marching form of
+ * lb_set_launch) or 128 (the default: marching or 24-row tiles, whichever is
+ * expected to be faster); seg_rows 0 gives every instance a share of one full
+ * wave proportional to its cells. */
 int lb_batch_set_launch(lb_batch* b, int block_x, int seg_rows);
 
 /* Persistent mode (the batched boiling curve of Sec. 3.2-3.3 in one launch

@@ -1,4 +1,4 @@
-// What the fused step uses beside a cell's arithmetic: the
+// What the forms of the fused step share beside a cell's arithmetic: the
 // pulled loads, the wall heat flux and its fold, shared-memory checks.
 #pragma once
 
@@ -63,7 +63,9 @@ __device__ __forceinline__ P2 sel(bool c, P2 a, P2 b) { return P2(c ? a.x() : b.
 // q(t) of the previous step: its columns' terms (P.qprev) summed in an order
 // that no launch shape changes and added to the statistics; by one warp. A
 // step writes its own terms and folds its predecessor's, off its critical
-// path (a fold kernel follows the last step of a call).
+// path (a fold kernel follows the last step of a call): folding inside the
+// step that made the terms took a counter, two fences and three trips to L2
+// after the slowest block, 2.2 us of the 6.9 us of a 100 x 100 step.
 __device__ __forceinline__ void fold_heat(const StepParams& P, const int lane) {
     double s[4] = {0.0, 0.0, 0.0, 0.0};
     for (int x = lane; x < P.Lx; x += 512) {  // 16 loads in flight

@@ -11,7 +11,9 @@
 namespace lbgpu {
 
 constexpr int HALO = 5;    // x-halo columns per side recomputed by a block
-constexpr int TILE_COLS = 54;    // columns of a strip (64 less the halos); a block owns two
+constexpr int TILE_COLS = 54;    // columns of a strip (64 less the halos); the marching form's blocks own two
+constexpr int TILE16_ROWS = 6;   // rows a tile of 16 / 24 computed rows writes
+constexpr int TILE24_ROWS = 14;
 
 enum { BC_WALLS = 0, BC_TOP_OUTFLOW = 1, BC_PERIODIC = 2 };
 enum : unsigned { ERR_EOS = 1u, ERR_NONFINITE = 2u, ERR_BOUNDS = 4u, ERR_TIMEOUT = 8u };

@@ -305,25 +305,66 @@ StepParams step_params(const lb_handle* h, const StepParams& base, int cur) {
 
 inline int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
 
-// Column strips of a step's blocks.
-inline int form_strips(int form, int Lx) {
-    (void)form;
-    return ceil_div(Lx, 2 * TILE_COLS);
+// Column strips and most rows of one pass of a form's block.
+inline int form_strips(int form, int Lx) { return ceil_div(Lx, form == FORM_MARCH ? 2 * TILE_COLS : TILE_COLS); }
+inline int form_rows(int form) { return form == FORM_TILE16 ? TILE16_ROWS : form == FORM_TILE24 ? TILE24_ROWS : INT32_MAX; }
+
+// About how long a step of `blocks` blocks of seg_rows rows takes, in us, on
+// nsm SMs that hold occ blocks each: the forms' measured times. A tile takes
+// the same time whatever its SM's neighbours do, wave after wave; a marching
+// block takes its rows plus the pipeline's ten, two per iteration, and its
+// iterations hardly lengthen until the SM's four blocks are there.
+double form_us(int form, long long blocks, int seg_rows, int nsm, int occ) {
+    const long long waves = ceil_div(blocks, (long long)nsm * occ);
+    if (form == FORM_TILE16) return 0.5 + 4.1 * waves * ceil_div(seg_rows, TILE16_ROWS);
+    if (form == FORM_TILE24) return 0.8 + 5.7 * waves * ceil_div(seg_rows, TILE24_ROWS);
+    const double per_sm = std::min((double)occ, (double)blocks / nsm);
+    return 1.0 + waves * ceil_div(seg_rows + 2 * HALO, 2) * (1.75 + 0.13 * per_sm);
 }
 
-// The launch shape of the fused step for this grid (seg_rows 0: segments that
-// fill the GPU once).
+// The launch shape of one form for this grid (seg_rows 0: automatic): a tile
+// form's tiles as equal as they come, marching segments that fill the GPU
+// once.
+int form_launch(int form, const lb_grid& g, int seg_rows, int nsm, Launch* out, int* occ) {
+    int threads = 0;
+    LB_CUDA(step_occupancy(form, &threads, occ), "occupancy");
+    if (*occ < 1) return fail(LB_E_INVAL, "the fused step's block of %d threads does not fit on an SM", threads);
+    out->form = form;
+    out->block_x = threads;
+    out->nstrips = form_strips(form, g.Lx);
+    int seg = seg_rows;
+    if (seg <= 0) {
+        if (form == FORM_MARCH) seg = std::max(8, ceil_div(g.Ly, std::max(1, nsm * *occ / out->nstrips)));
+        else seg = ceil_div(g.Ly, ceil_div(g.Ly, form_rows(form)));
+    }
+    out->seg_rows = seg;
+    out->nseg = ceil_div(g.Ly, seg);
+    return LB_OK;
+}
+
+// The launch shape of the fused step for this grid. block_x names the form
+// (64: marching, 128: tiles of 24 rows, 256: tiles of 16 rows); 0 takes the
+// one with the shortest estimate.
 int compute_launch(const lb_handle* h, int block_x, int seg_rows, Launch* out) {
-    int dev = 0, nsm = 0, occ = 0, threads = 0;
+    int dev = 0, nsm = 0, occ = 0;
     LB_CUDA(cudaGetDevice(&dev), "cudaGetDevice");
     LB_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev), "cudaDeviceGetAttribute");
     if (block_x != 0 && block_x != 64 && block_x != 128 && block_x != 256)
         return fail(LB_E_INVAL, "the fused step takes block_x 64, 128 or 256, not %d", block_x);
-    LB_CUDA(step_occupancy(FORM_MARCH, &threads, &occ), "occupancy");
-    if (occ < 1) return fail(LB_E_INVAL, "the fused step's block of %d threads does not fit on an SM", threads);
-    const int nstrips = form_strips(FORM_MARCH, h->grid.Lx);
-    const int seg = seg_rows > 0 ? seg_rows : std::max(8, ceil_div(h->grid.Ly, std::max(1, nsm * occ / nstrips)));
-    *out = Launch{FORM_MARCH, threads, seg, nstrips, ceil_div(h->grid.Ly, seg)};
+    if (block_x > 0)
+        return form_launch(block_x == 64 ? FORM_MARCH : block_x == 128 ? FORM_TILE24 : FORM_TILE16, h->grid, seg_rows, nsm,
+                           out, &occ);
+    double best = 0;
+    for (int form = 0; form < FORM_COUNT; ++form) {
+        Launch L;
+        const int rc = form_launch(form, h->grid, seg_rows, nsm, &L, &occ);
+        if (rc) return rc;
+        const double us = form_us(form, (long long)L.nstrips * L.nseg, L.seg_rows, nsm, occ);
+        if (form == 0 || us < best) {
+            best = us;
+            *out = L;
+        }
+    }
     return LB_OK;
 }
 
@@ -976,7 +1017,7 @@ size_t batch_tail_offset(const lb_batch_desc* d, int n, std::vector<size_t>* off
 long long batch_max_tiles(const lb_batch_desc* d, int n) {
     long long t = 0;
     for (int i = 0; i < n; ++i)
-        t += (long long)form_strips(FORM_MARCH, d[i].grid.Lx) * d[i].grid.Ly;
+        t += (long long)form_strips(FORM_TILE24, d[i].grid.Lx) * d[i].grid.Ly;
     return t;
 }
 
@@ -1016,8 +1057,8 @@ void batch_constants(lb_batch* b) {
         if (!same_constants(h->base, b->kconst)) b->kshared = false;
 }
 
-// Rows per tile in a batch whose tiles fit in `cap` slots, and how many tiles
-// that makes. Without a
+// Rows per tile of a form in a batch whose tiles fit in `cap` slots (and in
+// the tile form's own height), and how many tiles that makes. Without a
 // requested height every tile gets about the same number of rows: a block
 // costs its rows (plus the pipeline's halo) whatever share of its columns the
 // instance fills, and the step lasts as long as its longest tile.
@@ -1031,7 +1072,8 @@ int batch_height(const lb_batch* b, int form, long long cap, long long* tiles) {
     if (S <= 0) {
         int hi = 8;
         for (lb_handle* h : b->inst) hi = std::max(hi, h->grid.Ly);
-        S = 8;
+        hi = std::min(hi, form_rows(form));
+        S = std::min(8, hi);
         while (S < hi) {  // the smallest height whose tiles fit (tiles_at falls as the height grows)
             const int mid = S + (hi - S) / 2;
             if (tiles_at(mid) <= cap) hi = mid;
@@ -1042,10 +1084,11 @@ int batch_height(const lb_batch* b, int form, long long cap, long long* tiles) {
     return S;
 }
 
-// Per-instance segment height and block offsets. With an automatic
+// Form, per-instance segment height and block offsets. With an automatic
 // segment height the tiles of all instances are about equal and fill one wave
 // (tpb waves in the persistent mode, whose grid is one wave that takes about
-// tpb tiles per block).
+// tpb tiles per block). block_x 64 asks for the marching form; 128 takes the
+// form with the shortest estimate.
 int batch_layout(lb_batch* b) {
     const int n = (int)b->inst.size();
     int dev = 0, nsm = 0, occ = 0, S = 0;
@@ -1053,11 +1096,22 @@ int batch_layout(lb_batch* b) {
     LB_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev), "cudaDeviceGetAttribute");
     batch_constants(b);
     const int waves = std::max(1, b->tpb);
-    b->form = FORM_MARCH;
-    LB_CUDA(batch_occupancy(b->form, b->kshared, b->tpb > 0, &b->threads, &occ), "occupancy");
-    if (occ < 1) return fail(LB_E_INVAL, "the batched step's block of %d threads does not fit on an SM", b->threads);
-    long long tiles = 0;
-    S = batch_height(b, b->form, (long long)nsm * occ * waves, &tiles);
+    double best = 0;
+    for (int form : {FORM_MARCH, FORM_TILE24}) {
+        if (form != FORM_MARCH && b->block_x == 64) continue;
+        int threads = 0, o = 0;
+        LB_CUDA(batch_occupancy(form, b->kshared, b->tpb > 0, &threads, &o), "occupancy");
+        if (o < 1) return fail(LB_E_INVAL, "the batched step's block of %d threads does not fit on an SM", threads);
+        long long tiles = 0;
+        const int height = batch_height(b, form, (long long)nsm * o * waves, &tiles);
+        const double us = form_us(form, tiles, height, nsm, o);
+        if (form != FORM_MARCH && us >= best) continue;
+        best = us;
+        b->form = form;
+        b->threads = threads;
+        occ = o;
+        S = height;
+    }
     b->h_off.assign(n + 1, 0);
     for (int i = 0; i < n; ++i) {
         lb_handle* h = b->inst[i];

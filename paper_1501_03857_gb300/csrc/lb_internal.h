@@ -8,8 +8,8 @@
 
 namespace lbgpu {
 
-// Forms of the fused step (lb_march.cuh).
-enum Form { FORM_MARCH = 0, FORM_COUNT = 1 };
+// Forms of the fused step (lb_march.cuh, lb_tile.cuh).
+enum Form { FORM_MARCH = 0, FORM_TILE16 = 1, FORM_TILE24 = 2, FORM_COUNT = 3 };
 
 // Launch shape of the fused step: nstrips x nseg blocks of seg_rows rows
 // each; block_x threads per block (the form's).
@@ -43,7 +43,8 @@ cudaError_t recompute_prepare();
 cudaError_t launch_recompute(const StepParams& P, const RecomputeOut& R, bool out, bool heat, bool fold,
                              const Launch& L, cudaStream_t st);
 
-// The same step over a table of independent instances in one launch ; instance i owns blocks
+// The same step over a table of independent instances in one launch (the
+// marching form and the 24-row tiles); instance i owns blocks
 // [block_off[i], block_off[i+1]).
 cudaError_t batch_prepare();
 cudaError_t batch_occupancy(int form, bool shared_k, bool persistent, int* threads, int* blocks_per_sm);

@@ -1,4 +1,5 @@
-// The fused step as a march up column strips.
+// The marching form of the fused step (the other is lb_tile.cuh): for domains
+// that fill the GPU.
 //
 // A block of 64 threads owns two adjacent strips of 54 columns and a segment
 // of rows, thread lc the column lc of both (5 halo columns per side), and

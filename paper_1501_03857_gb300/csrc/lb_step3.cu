@@ -1,5 +1,9 @@
 // The fused time step of one domain: stream + collide + forces, RK4
-// temperature, wall heat flux, in one kernel (lb_march.cuh).
+// temperature, wall heat flux, in one kernel. It has two forms with the same
+// arithmetic per cell (lb_cell.cuh) and so the same results bit for bit: a
+// marching one for domains that fill the GPU (lb_march.cuh) and a tiled one
+// for smaller ones (lb_tile.cuh, two tile heights); the host picks by the
+// measured times of each (pick_form in lb_host.cu).
 #include "lb_forms.cuh"
 
 namespace lbgpu {
@@ -8,11 +12,13 @@ namespace {
 
 template <class F>
 __global__ void __launch_bounds__(F::threads, F::min_blocks) lb_step_kernel(const StepParams P, const int fold) {
+    grid_start();
     F::template body<false, false, true, true>(P, P, blockIdx.x, fold, nullptr);
 }
 
 // q(t) of the last step of a call (fold_heat): one warp.
 __global__ void __launch_bounds__(32) lb_fold_kernel(const StepParams P) {
+    grid_start();
     fold_heat(P, threadIdx.x);
 }
 

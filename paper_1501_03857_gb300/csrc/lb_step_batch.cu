@@ -1,6 +1,7 @@
 // Many independent simulations in one launch (the boiling-curve batch): one
 // launch per step, or one cooperative launch for a run of steps. The
-// marching form of the fused step (lb_march.cuh).
+// marching form and the taller tiles of the fused step (lb_march.cuh,
+// lb_tile.cuh).
 #include "lb_forms.cuh"
 
 namespace lbgpu {
@@ -41,6 +42,7 @@ __global__ void __launch_bounds__(F::threads, F::min_blocks)
     lb_step_batch(const StepParams K, const StepParams* __restrict__ table, const int* __restrict__ block_off, const int n,
                   const int fold) {
     __shared__ StepParams sP;
+    grid_start();
     const int b = batch_instance<F::threads>(table, block_off, n, sP);
     F::template body<false, false, true, true>(sP, SK ? K : sP, b, fold, nullptr);
 }
@@ -48,6 +50,7 @@ __global__ void __launch_bounds__(F::threads, F::min_blocks)
 // q(t) of every instance's last step of a call: one warp per instance, from
 // the parameters of the step that would follow.
 __global__ void __launch_bounds__(32) lb_batch_fold(const StepParams* __restrict__ table) {
+    grid_start();
     if (table[blockIdx.x].bc != BC_PERIODIC) fold_heat(table[blockIdx.x], threadIdx.x);
 }
 
@@ -207,14 +210,15 @@ struct BatchForm {
 
 template <class F>
 auto with_batch_form(int form, F f) {
-    (void)form;
+    if (form == FORM_TILE24) return f(Tile24{});
     return f(MarchForm{});
 }
 
 }  // namespace
 
 cudaError_t batch_prepare() {
-    return BatchForm<MarchForm>::prepare();
+    cudaError_t e = BatchForm<MarchForm>::prepare();
+    return e == cudaSuccess ? BatchForm<Tile24>::prepare() : e;
 }
 
 cudaError_t batch_occupancy(int form, bool shared_k, bool persistent, int* threads, int* n) {
