@@ -1,5 +1,7 @@
 // Off-hot-path kernels: initial state, macroscopic fields, FP64 mass sum,
 // and the pressure probe run after a step when probes are set (Fig. 3).
+#include <algorithm>
+
 #include "lb_internal.h"
 
 namespace lbgpu {
@@ -97,25 +99,141 @@ __global__ void macro_pass2(const StepParams P, const float* __restrict__ scr, f
     for (int y = blockIdx.y; y < P.Ly; y += gridDim.y) macro2_cell(P, scr, orho, oux, ouy, oT, ostride, x, y);
 }
 
-__global__ void mass_kernel(const StepParams P, const float* __restrict__ f) {
-    __shared__ double red[32];
-    double s = 0.0;
-    const long long n = 9LL * P.Ly * P.Lx;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
-         k += (long long)gridDim.x * blockDim.x) {
-        const long long a = k / ((long long)P.Ly * P.Lx);
-        const long long rem = k - a * P.Ly * P.Lx;
-        const int y = (int)(rem / P.Lx), x = (int)(rem - (long long)y * P.Lx);
-        s += (double)f[a * P.plane + (long long)y * P.pitch + x];
+// The fields of lb_fields in one pass (launch_fields): a block of FIELD_T
+// threads marches up a segment of rows, one column per thread, the outer two
+// halo. psi of the last rows sits in a four-row shared ring (one barrier per
+// row); rho and the momentum sums of a row wait in registers for the row
+// above it. Bound by HBM: ten planes in, four out, against 48 more bytes per
+// cell when rho, psi and j went through scratch planes between two kernels.
+constexpr int FIELD_T = 128, FIELD_COLS = FIELD_T - 2, FIELD_ROWS = 16;
+
+__global__ void __launch_bounds__(FIELD_T) fields_kernel(const StepParams P, float* __restrict__ orho,
+                                                         float* __restrict__ oux, float* __restrict__ ouy,
+                                                         float* __restrict__ oT, int ostride) {
+    __shared__ float ring[4][FIELD_T];
+    const int Lx = P.Lx, Ly = P.Ly;
+    const bool periodic = P.bc == BC_PERIODIC;
+    const int lc = threadIdx.x;
+    const int nstrips = (Lx + FIELD_COLS - 1) / FIELD_COLS;
+    const int x0 = blockIdx.x % nstrips * FIELD_COLS;
+    const int ys = blockIdx.x / nstrips * FIELD_ROWS, ye = min(ys + FIELD_ROWS, Ly);
+    const int x = wrap(x0 - 1 + lc, Lx);
+    const int xm = x == 0 ? Lx - 1 : x - 1, xp = x == Lx - 1 ? 0 : x + 1;
+    const bool own = lc >= 1 && lc <= FIELD_COLS && x0 + lc - 1 < Lx;
+    const int lo = periodic ? ys - 1 : max(ys - 1, 0), hi = periodic ? ye : min(ye, Ly - 1);  // psi rows
+    bool bad = false;
+    float rho = 0.f, jx = 0.f, jy = 0.f, th = 0.f;  // row r
+    for (int L = lo; L <= hi + 1; ++L) {
+        const float rho1 = rho, jx1 = jx, jy1 = jy, th1 = th;  // row L - 1
+        if (L <= hi) {
+            const int y = periodic ? wrap(L, Ly) : L;
+            float f[9];
+            load_row(P, y, x, xm, xp, f, th);
+            wall_fill(P, y, f);
+            rho = 0.f;
+#pragma unroll
+            for (int a = 0; a < 9; ++a) rho += f[a];
+            jx = (f[1] - f[3]) + (f[5] - f[6]) + (f[8] - f[7]);
+            jy = (f[2] - f[4]) + (f[5] + f[6]) - (f[7] + f[8]);
+            ring[L & 3][lc] = eos_psi(rho, P.Ts + th, P, bad);
+        }
+        __syncthreads();
+        const int r = L - 1;
+        if (r >= ys && r < ye && own) {
+            const bool wall = !periodic && (r == 0 || r == Ly - 1);
+            const float* pc = &ring[r & 3][lc];
+            const float ps = *pc;
+            float Fx = 0.f, Fy = 0.f;
+            if (!wall || P.ghost) {  // the ghost row beyond a wall copies the wall row
+                const float* pm = wall && r == 0 ? pc : &ring[(r - 1) & 3][lc];
+                const float* pn = wall && r == Ly - 1 ? pc : &ring[(r + 1) & 3][lc];
+                float sx, sy;
+                psi_sum(pm, pc, pn, sx, sy);
+                Fx = -P.G * ps * sx;
+                Fy = -P.G * ps * sy;
+            }
+            if (!wall) {
+                if (!periodic && r == 1) Fy += P.gw6 * ps * ps;
+                Fy -= P.g * (rho1 - P.rho_ave);
+            }
+            const int o = r * ostride + x;
+            if (orho) orho[o] = rho1;
+            if (oux) oux[o] = (jx1 + 0.5f * Fx) / rho1;
+            if (ouy) ouy[o] = (jy1 + 0.5f * Fy) / rho1;
+            if (oT) oT[o] = P.Ts + th1;
+        }
+    }
+    if (bad) atomicOr(&P.acc->err, ERR_EOS);
+}
+
+// Sums of a few dozen floats without rounding, in FP32: a value is cut into
+// multiples of 2^-8, of 2^-23 and the rest by adding and subtracting a power
+// of two (extraction, as in Rump, Ogita and Oishi, "Accurate floating-point
+// summation", SIAM J. Sci. Comput. 31, 2008), and each part's sum stays
+// within 24 bits: exact for up to 64 values with 2^-18 <= |v| < 2^9 or v = 0.
+// FP64 adds only the parts' sums.
+struct Parts {
+    float hi, mid, lo;
+    bool ok;  // every value was in that range
+    __device__ __forceinline__ void clear() {
+        hi = mid = lo = 0.f;
+        ok = true;
+    }
+    __device__ __forceinline__ void add(float v) {
+        constexpr float c1 = 49152.f, c2 = 1.5f;  // 1.5 x 2^15, 1.5 x 2^0
+        const float h = __fadd_rn(__fadd_rn(v, c1), -c1);
+        const float r = __fadd_rn(v, -h);
+        const float m = __fadd_rn(__fadd_rn(r, c2), -c2);
+        hi = __fadd_rn(hi, h);
+        mid = __fadd_rn(mid, m);
+        lo = __fadd_rn(lo, __fadd_rn(r, -m));
+        const unsigned u = __float_as_uint(v) & 0x7fffffffu;
+        ok &= u - 0x36800000u < 0x44000000u - 0x36800000u || u == 0u;
+    }
+    __device__ __forceinline__ double sum() const { return ((double)lo + (double)mid) + (double)hi; }
+};
+
+// Sum of f over the cells and directions, exact up to the FP64 sum of runs of
+// 64 values. Warps take rows of the nine planes, four columns per lane and
+// load. FP64 adds run at 1/64 of the FP32 rate: one per value took 154 us on
+// 2048^2 (22 us from HBM), one per run of 64 takes the figure of the read.
+__global__ void __launch_bounds__(256) mass_kernel(const StepParams P, const float* __restrict__ f) {
+    __shared__ double red[8];
+    double t = 0.0;
+    const int lane = threadIdx.x & 31;
+    const int rows = 9 * P.Ly;  // of pitch floats, pitch a multiple of 32: 16-byte aligned
+    for (int r = blockIdx.x * 8 + (threadIdx.x >> 5); r < rows; r += gridDim.x * 8) {
+        const float* p = f + (size_t)r * P.pitch;
+        for (int x0 = 4 * lane; x0 < P.Lx; x0 += 16 * 128) {
+            const int n = min(16, (P.Lx - x0 + 127) / 128);
+            Parts s;
+            s.clear();
+#pragma unroll 4
+            for (int k = 0; k < n; ++k) {
+                const int x = x0 + 128 * k;
+                const float4 v = __ldg(reinterpret_cast<const float4*>(p + x));
+                s.add(v.x);
+                s.add(x + 1 < P.Lx ? v.y : 0.f);
+                s.add(x + 2 < P.Lx ? v.z : 0.f);
+                s.add(x + 3 < P.Lx ? v.w : 0.f);
+            }
+            if (s.ok) {
+                t += s.sum();
+            } else {
+                for (int k = 0; k < n; ++k)
+                    for (int j = 0; j < 4; ++j)
+                        if (x0 + 128 * k + j < P.Lx) t += (double)p[x0 + 128 * k + j];
+            }
+        }
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (lane == 0) red[threadIdx.x >> 5] = t;
     __syncthreads();
     if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-        atomicAdd(&P.acc->mass, t);
+        double m = 0.0;
+        for (int w = 0; w < 8; ++w) m += red[w];
+        atomicAdd(&P.acc->mass, m);
     }
 }
 
@@ -137,10 +255,17 @@ cudaError_t launch_macro(const StepParams& P, float* scratch, float* rho, float*
     return cudaGetLastError();
 }
 
+cudaError_t launch_fields(const StepParams& P, float* rho, float* ux, float* uy, float* T, int ostride,
+                          cudaStream_t st) {
+    const int nstrips = (P.Lx + FIELD_COLS - 1) / FIELD_COLS, nseg = (P.Ly + FIELD_ROWS - 1) / FIELD_ROWS;
+    fields_kernel<<<nstrips * nseg, FIELD_T, 0, st>>>(P, rho, ux, uy, T, ostride);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_mass(const StepParams& P, const float* f, cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(&P.acc->mass, 0, sizeof(double), st);
     if (e != cudaSuccess) return e;
-    mass_kernel<<<256, 256, 0, st>>>(P, f);
+    mass_kernel<<<std::min(8 * 152, (9 * P.Ly + 7) / 8), 256, 0, st>>>(P, f);
     return cudaGetLastError();
 }
 

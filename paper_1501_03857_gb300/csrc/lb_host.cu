@@ -718,12 +718,12 @@ int lb_fields(lb_handle* h, float* rho, float* ux, float* uy, float* T, int on_d
     const int Lx = h->grid.Lx, Ly = h->grid.Ly, pitch = h->lay.pitch;
     const size_t pl = h->lay.plane;
     if (on_device) {
-        LB_CUDA(launch_macro(P, scr, rho, ux, uy, T, Lx, h->st), "fields kernel");
+        LB_CUDA(launch_fields(P, rho, ux, uy, T, Lx, h->st), "fields kernel");
         return check_device_errors(h);
     }
-    float* o[4] = {rho ? scr + 4 * pl : nullptr, ux ? scr + 5 * pl : nullptr, uy ? scr + 6 * pl : nullptr,
-                   T ? scr + 7 * pl : nullptr};
-    LB_CUDA(launch_macro(P, scr, o[0], o[1], o[2], o[3], pitch, h->st), "fields kernel");
+    float* o[4] = {rho ? scr : nullptr, ux ? scr + pl : nullptr, uy ? scr + 2 * pl : nullptr,
+                   T ? scr + 3 * pl : nullptr};
+    LB_CUDA(launch_fields(P, o[0], o[1], o[2], o[3], pitch, h->st), "fields kernel");
     float* dst[4] = {rho, ux, uy, T};
     for (int k = 0; k < 4; ++k)
         if (dst[k])

@@ -78,8 +78,14 @@ cudaError_t persist_launch(int form, const StepParams* K, const PersistArgs& A, 
 // rows at their Dirichlet values. rho0 is pitched [Ly][pitch].
 cudaError_t launch_init(const StepParams& P, const float* rho0, float* f, float* th, cudaStream_t st);
 
-// Macroscopic fields (rho, u with the level's forces, T) into outputs with
-// row stride ostride; scratch holds 4 pitched planes.
+// Macroscopic fields (rho, u with the level's forces, T; any may be null)
+// into outputs with row stride ostride that overlap neither the populations
+// nor theta.
+cudaError_t launch_fields(const StepParams& P, float* rho, float* ux, float* uy, float* T, int ostride,
+                          cudaStream_t st);
+
+// The same in two kernels through scratch (4 pitched planes), after which the
+// populations are no longer read: for callers whose outputs may overlay them.
 cudaError_t launch_macro(const StepParams& P, float* scratch, float* rho, float* ux, float* uy,
                          float* T, int ostride, cudaStream_t st);
 
