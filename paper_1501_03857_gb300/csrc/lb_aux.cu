@@ -1,6 +1,7 @@
 // Off-hot-path kernels: initial state, macroscopic fields, FP64 mass sum,
 // and the pressure probe run after a step when probes are set (Fig. 3).
 #include <algorithm>
+#include <type_traits>
 
 #include "lb_internal.h"
 
@@ -166,6 +167,31 @@ __global__ void __launch_bounds__(FIELD_T) fields_kernel(const StepParams P, flo
     if (bad) atomicOr(&P.acc->err, ERR_EOS);
 }
 
+// Rows of lx floats between arrays of row stride sp and dp, two arrays (the
+// populations' 9 Ly rows, theta's Ly) in one launch; V floats per access. A
+// warp takes 4 KB runs of a row, so that short rows do not leave lanes idle
+// for long and long ones keep many loads in flight.
+template <int V>
+__global__ void __launch_bounds__(256) copy_rows(const float* __restrict__ s0, float* __restrict__ d0, int n0,
+                                                 const float* __restrict__ s1, float* __restrict__ d1, int n1, int lx,
+                                                 int sp, int dp) {
+    using T = typename std::conditional<V == 4, float4, float>::type;
+    constexpr int RUN = 1024;  // floats
+    const int lane = threadIdx.x & 31;
+    const int runs = (lx + RUN - 1) / RUN;
+    const long long total = (long long)(n0 + n1) * runs;
+    for (long long w = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); w < total; w += (long long)gridDim.x * 8) {
+        const int r = (int)(w / runs), x0 = (int)(w - (long long)r * runs) * RUN;
+        const bool second = r >= n0;
+        const float* s = (second ? s1 + (size_t)(r - n0) * sp : s0 + (size_t)r * sp) + x0;
+        float* d = (second ? d1 + (size_t)(r - n0) * dp : d0 + (size_t)r * dp) + x0;
+        const int n = min(RUN, lx - x0) / V;
+#pragma unroll 8
+        for (int i = lane; i < n; i += 32)
+            reinterpret_cast<T*>(d)[i] = __ldg(reinterpret_cast<const T*>(s) + i);
+    }
+}
+
 // Sums of a few dozen floats without rounding, in FP32: a value is cut into
 // multiples of 2^-8, of 2^-23 and the rest by adding and subtracting a power
 // of two (extraction, as in Rump, Ogita and Oishi, "Accurate floating-point
@@ -252,6 +278,36 @@ cudaError_t launch_macro(const StepParams& P, float* scratch, float* rho, float*
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     macro_pass2<<<grid, 128, 0, st>>>(P, scratch, rho, ux, uy, T, ostride);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_copy_state(const float* f_src, float* f_dst, const float* t_src, float* t_dst, int Lx, int Ly,
+                              int src_pitch, int dst_pitch, cudaStream_t st) {
+    const int n0 = f_src ? 9 * Ly : 0, n1 = t_src ? Ly : 0;
+    const uintptr_t all = (uintptr_t)f_src | (uintptr_t)f_dst | (uintptr_t)t_src | (uintptr_t)t_dst;
+    const long long warps = (long long)(n0 + n1) * ((Lx + 1023) / 1024);
+    const int blocks = (int)std::min<long long>((warps + 7) / 8, 16 * 152);
+    if (blocks == 0) return cudaSuccess;
+    // (the pitch is a multiple of 32 floats: the other side's rows decide)
+    if (all % 16 == 0 && Lx % 4 == 0)
+        copy_rows<4><<<blocks, 256, 0, st>>>(f_src, f_dst, n0, t_src, t_dst, n1, Lx, src_pitch, dst_pitch);
+    else
+        copy_rows<1><<<blocks, 256, 0, st>>>(f_src, f_dst, n0, t_src, t_dst, n1, Lx, src_pitch, dst_pitch);
+    return cudaGetLastError();
+}
+
+// The accumulator records of a batch's instances into out (host memory the
+// device can write), one thread each; reset clears the heat-flux sums.
+__global__ void collect_acc(const StepParams* __restrict__ table, int n, Acc* out, int reset) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    Acc* a = table[i].acc;
+    out[i] = *a;
+    if (reset) a->q_sum = a->q_sum2 = a->q_n = 0.0;
+}
+
+cudaError_t launch_collect(const StepParams* table, int n, Acc* out, bool reset, cudaStream_t st) {
+    collect_acc<<<(n + 63) / 64, 64, 0, st>>>(table, n, out, reset ? 1 : 0);
     return cudaGetLastError();
 }
 

@@ -212,7 +212,8 @@ struct lb_handle {
     int64_t steps;
     Launch launch;
     StepParams base;
-    float* wall_pinned;      // pinned staging of theta_b(x) for the upload
+    Acc* rec;                // pinned: the accumulator record as last read
+    float* wall_pinned;      // pinned staging of theta_b(x) for the upload (follows rec)
     cudaEvent_t wall_done;   // the last upload from wall_pinned has run
     bool wall_pending;
     // adjoint: private stream for captured segment graphs, keyed by
@@ -398,11 +399,30 @@ int report_device_errors(lb_handle* h, unsigned err) {
     return LB_OK;
 }
 
-int check_device_errors(lb_handle* h) {
-    unsigned err = 0;
+// The accumulator record into h->rec, after everything issued on the stream:
+// one copy to pinned memory and one wait (a read into pageable memory waits
+// once more).
+int read_acc(lb_handle* h) {
+    LB_CUDA(cudaMemcpyAsync(h->rec, h->acc, sizeof(Acc), cudaMemcpyDeviceToHost, h->st), "read accumulators");
     LB_CUDA(cudaStreamSynchronize(h->st), "cudaStreamSynchronize");
-    LB_CUDA(cudaMemcpy(&err, &h->acc->err, sizeof(unsigned), cudaMemcpyDeviceToHost), "read error flags");
-    return report_device_errors(h, err);
+    return LB_OK;
+}
+
+int check_device_errors(lb_handle* h) {
+    const int rc = read_acc(h);
+    return rc ? rc : report_device_errors(h, h->rec->err);
+}
+
+// Whether p is memory of the current device (else copies go through
+// cudaMemcpy, which takes any address).
+bool on_this_device(const void* p) {
+    cudaPointerAttributes a;
+    int dev = -1;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == dev;
 }
 
 int upload_wall(lb_handle* h) {
@@ -433,7 +453,7 @@ void release(lb_handle* h) {
     if (h->adj_stream) cudaStreamDestroy(h->adj_stream);
     if (h->wall_pending) cudaEventSynchronize(h->wall_done);
     if (h->wall_done) cudaEventDestroy(h->wall_done);
-    if (h->wall_pinned) cudaFreeHost(h->wall_pinned);
+    if (h->rec) cudaFreeHost(h->rec);
     delete h;
 }
 
@@ -604,6 +624,7 @@ int lb_init(lb_handle** out, const lb_grid* grid, const lb_eos* eos, const lb_th
     h->cur = 0;
     h->st = (cudaStream_t)stream;
     h->steps = 0;
+    h->rec = nullptr;
     h->wall_pinned = nullptr;
     h->wall_done = nullptr;
     h->wall_pending = false;
@@ -612,7 +633,8 @@ int lb_init(lb_handle** out, const lb_grid* grid, const lb_eos* eos, const lb_th
     h->adj_stream2 = nullptr;
     h->adj_ready[0] = h->adj_ready[1] = h->adj_free[0] = h->adj_free[1] = nullptr;
     {
-        cudaError_t e0 = cudaMallocHost((void**)&h->wall_pinned, grid->Lx * sizeof(float));
+        cudaError_t e0 = cudaMallocHost((void**)&h->rec, sizeof(Acc) + grid->Lx * sizeof(float));
+        if (e0 == cudaSuccess) h->wall_pinned = (float*)(h->rec + 1);
         if (e0 == cudaSuccess) e0 = cudaEventCreateWithFlags(&h->wall_done, cudaEventDisableTiming);
         if (e0 != cudaSuccess) {
             release(h);
@@ -688,13 +710,9 @@ int lb_set_wettability(lb_handle* h, double Gw) {
     return LB_OK;
 }
 
-int lb_heat_flux(lb_handle* h, double* q_inst, double* q_mean, double* q_std, int64_t* nsamples, int reset) {
-    if (!h) return fail(LB_E_INVAL, "null handle");
-    Acc a;
-    // one read of the accumulator record, fault flags included
-    LB_CUDA(cudaMemcpyAsync(&a, h->acc, sizeof(Acc), cudaMemcpyDeviceToHost, h->st), "read accumulators");
-    LB_CUDA(cudaStreamSynchronize(h->st), "cudaStreamSynchronize");
-    int rc = report_device_errors(h, a.err);
+// The heat-flux statistics of an accumulator record into outputs that may be
+// null.
+static void flux_stats(const Acc& a, double* q_inst, double* q_mean, double* q_std, int64_t* nsamples) {
     const double n = a.q_n;
     const double mean = n > 0 ? a.q_sum / n : 0.0;
     const double var = n > 1 ? std::max(0.0, (a.q_sum2 - n * mean * mean) / (n - 1)) : 0.0;
@@ -702,10 +720,18 @@ int lb_heat_flux(lb_handle* h, double* q_inst, double* q_mean, double* q_std, in
     if (q_mean) *q_mean = mean;
     if (q_std) *q_std = std::sqrt(var);
     if (nsamples) *nsamples = (int64_t)n;
-    if (reset) {
-        LB_CUDA(cudaMemsetAsync(&h->acc->q_sum, 0, 3 * sizeof(double), h->st), "reset accumulators");
-        LB_CUDA(cudaStreamSynchronize(h->st), "cudaStreamSynchronize");
-    }
+}
+
+int lb_heat_flux(lb_handle* h, double* q_inst, double* q_mean, double* q_std, int64_t* nsamples, int reset) {
+    if (!h) return fail(LB_E_INVAL, "null handle");
+    // one read of the accumulator record, fault flags included; the reset
+    // follows it in stream order
+    int rc = read_acc(h);
+    if (rc) return rc;
+    const Acc a = *h->rec;
+    rc = report_device_errors(h, a.err);
+    flux_stats(a, q_inst, q_mean, q_std, nsamples);
+    if (reset) LB_CUDA(cudaMemsetAsync(&h->acc->q_sum, 0, 3 * sizeof(double), h->st), "reset accumulators");
     return rc;
 }
 
@@ -737,6 +763,12 @@ int lb_get_state(lb_handle* h, float* fpost, float* theta, int on_device) {
     if (!h) return fail(LB_E_INVAL, "null handle");
     const int Lx = h->grid.Lx, Ly = h->grid.Ly, pitch = h->lay.pitch;
     const cudaMemcpyKind k = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
+    if (on_device && (!fpost || on_this_device(fpost)) && (!theta || on_this_device(theta))) {
+        LB_CUDA(launch_copy_state(fpost ? h->f[h->cur] : nullptr, fpost, theta ? h->t[h->cur] : nullptr, theta, Lx, Ly,
+                                  pitch, Lx, h->st),
+                "state copy");
+        return check_device_errors(h);
+    }
     if (fpost)
         LB_CUDA(cudaMemcpy2DAsync(fpost, Lx * sizeof(float), h->f[h->cur], pitch * sizeof(float), Lx * sizeof(float),
                                   9 * Ly, k, h->st),
@@ -752,6 +784,10 @@ int lb_set_state(lb_handle* h, const float* fpost, const float* theta, int on_de
     if (!h) return fail(LB_E_INVAL, "null handle");
     const int Lx = h->grid.Lx, Ly = h->grid.Ly, pitch = h->lay.pitch;
     const cudaMemcpyKind k = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+    if (on_device && (!fpost || on_this_device(fpost)) && (!theta || on_this_device(theta))) {
+        LB_CUDA(launch_copy_state(fpost, h->f[h->cur], theta, h->t[h->cur], Lx, Ly, Lx, pitch, h->st), "state copy");
+        return LB_OK;
+    }
     if (fpost)
         LB_CUDA(cudaMemcpy2DAsync(h->f[h->cur], pitch * sizeof(float), fpost, Lx * sizeof(float), Lx * sizeof(float),
                                   9 * Ly, k, h->st),
@@ -768,8 +804,10 @@ int lb_mass(lb_handle* h, double* mass) {
     if (!h || !mass) return fail(LB_E_INVAL, "null argument");
     StepParams P = h->base;
     LB_CUDA(launch_mass(P, h->f[h->cur], h->st), "mass kernel");
-    LB_CUDA(cudaMemcpyAsync(mass, &h->acc->mass, sizeof(double), cudaMemcpyDeviceToHost, h->st), "mass read-back");
-    return check_device_errors(h);
+    const int rc = read_acc(h);
+    if (rc) return rc;
+    *mass = h->rec->mass;
+    return report_device_errors(h, h->rec->err);
 }
 
 int lb_sync(lb_handle* h) {
@@ -996,6 +1034,7 @@ struct lb_batch {
     std::vector<int> h_tile_off, h_ntiles;
     int pgrid;                   // blocks of the persistent launch
     cudaGraphExec_t pgraph;      // PERSIST_STEPS steps in one launch
+    Acc* rec;                    // pinned [n]: the instances' records as last read
 };
 
 namespace {
@@ -1294,6 +1333,7 @@ void batch_release(lb_batch* b) {
     if (b->ev_in) cudaEventDestroy(b->ev_in);
     if (b->ev_out) cudaEventDestroy(b->ev_out);
     if (b->gs) cudaStreamDestroy(b->gs);
+    if (b->rec) cudaFreeHost(b->rec);
     for (lb_handle* h : b->inst) release(h);
     delete b;
 }
@@ -1338,6 +1378,7 @@ int lb_batch_init(lb_batch** out, const lb_batch_desc* d, int n, void* dev_works
     b->d_tiles = nullptr;
     b->d_tile_off = b->d_ntiles = nullptr;
     b->d_arrive = nullptr;
+    b->rec = nullptr;
     char* ws = (char*)dev_workspace;
     const size_t tail = batch_tail_offset(d, n, &b->ws_off);
     for (int i = 0; i < n; ++i) {
@@ -1361,6 +1402,7 @@ int lb_batch_init(lb_batch** out, const lb_batch_desc* d, int n, void* dev_works
     b->d_arrive = (unsigned*)(ws + T.arrive);
     b->max_tiles = (int)std::min<long long>(batch_max_tiles(d, n), INT32_MAX);
     cudaError_t e = batch_prepare();
+    if (e == cudaSuccess) e = cudaMallocHost((void**)&b->rec, n * sizeof(Acc));
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->gs, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_in, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_out, cudaEventDisableTiming);
@@ -1445,15 +1487,18 @@ int lb_batch_step(lb_batch* b, int nsteps) {
     return LB_OK;
 }
 
-// Every instance is read (and its fault flags cleared); the first failure
+// Every instance's record in one launch and one wait (the instances one by one
+// took 20 us each); fault flags are cleared where set, and the first failure
 // is returned.
-int lb_batch_heat_flux(lb_batch* b, double* q_inst, double* q_mean, double* q_std, int64_t* nsamples, int reset) {
-    if (!b) return fail(LB_E_INVAL, "null batch");
+static int batch_read(lb_batch* b, bool reset) {
+    int rc = batch_upload(b);  // the table names the instances' records
+    if (rc) return rc;
+    LB_CUDA(launch_collect(b->table, (int)b->inst.size(), b->rec, reset, b->st), "read accumulators");
+    LB_CUDA(cudaStreamSynchronize(b->st), "cudaStreamSynchronize");
     int first = LB_OK;
     std::string msg;
     for (size_t i = 0; i < b->inst.size(); ++i) {
-        int rc = lb_heat_flux(b->inst[i], q_inst ? q_inst + i : nullptr, q_mean ? q_mean + i : nullptr,
-                              q_std ? q_std + i : nullptr, nsamples ? nsamples + i : nullptr, reset);
+        rc = report_device_errors(b->inst[i], b->rec[i].err);
         if (rc && first == LB_OK) {
             first = rc;
             msg = g_err;
@@ -1461,6 +1506,16 @@ int lb_batch_heat_flux(lb_batch* b, double* q_inst, double* q_mean, double* q_st
     }
     if (first) g_err = msg;
     return first;
+}
+
+int lb_batch_heat_flux(lb_batch* b, double* q_inst, double* q_mean, double* q_std, int64_t* nsamples, int reset) {
+    if (!b) return fail(LB_E_INVAL, "null batch");
+    const int rc = batch_read(b, reset != 0);
+    if (rc == LB_E_CUDA) return rc;
+    for (size_t i = 0; i < b->inst.size(); ++i)
+        flux_stats(b->rec[i], q_inst ? q_inst + i : nullptr, q_mean ? q_mean + i : nullptr, q_std ? q_std + i : nullptr,
+                   nsamples ? nsamples + i : nullptr);
+    return rc;
 }
 
 int lb_batch_get_state(lb_batch* b, int i, float* fpost, float* theta, int on_device) {
@@ -1500,17 +1555,7 @@ int lb_batch_info(lb_batch* b, int64_t* steps, int* block_x, int* nblocks) {
 
 int lb_batch_sync(lb_batch* b) {
     if (!b) return fail(LB_E_INVAL, "null batch");
-    int first = LB_OK;
-    std::string msg;
-    for (lb_handle* h : b->inst) {
-        int rc = check_device_errors(h);
-        if (rc && first == LB_OK) {
-            first = rc;
-            msg = g_err;
-        }
-    }
-    if (first) g_err = msg;
-    return first;
+    return batch_read(b, false);
 }
 
 int lb_batch_destroy(lb_batch* b) {

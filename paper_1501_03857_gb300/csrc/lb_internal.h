@@ -107,6 +107,15 @@ cudaError_t adjoint_reverse_step(const StepParams& P, const RecomputeOut& R, voi
 cudaError_t adjoint_grads_finish(const StepParams& P, void* work, const float* lt0, double* dTb_host,
                                  double* dGw_host, cudaStream_t st);
 
+// Populations (9 Ly rows) and theta (Ly rows) of Lx floats between device
+// arrays of different row strides; a null source is skipped.
+cudaError_t launch_copy_state(const float* f_src, float* f_dst, const float* t_src, float* t_dst, int Lx, int Ly,
+                              int src_pitch, int dst_pitch, cudaStream_t st);
+
+// The accumulator records of a batch's instances (table[i].acc) into out, in
+// pinned host memory; reset clears the heat-flux sums after reading.
+cudaError_t launch_collect(const StepParams* table, int n, Acc* out, bool reset, cudaStream_t st);
+
 // Record the message lb_last_error() returns on this thread.
 void set_last_error(const char* msg);
 
