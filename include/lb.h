@@ -282,13 +282,12 @@ int lb_batch_set_launch(lb_batch* b, int block_x, int seg_rows);
  * are cut into tiles (a block's column strips x a segment of rows;
  * with seg_rows 0 the segments give about tiles_per_block tiles per block),
  * the tiles are dealt out to the blocks (longest first to the least loaded
- * block), and a tile starts a step once every tile of its instance has
- * finished the previous one. Results are bit-identical to stepping each
- * instance alone. Each of those waits polls a
- * device counter at most wait_limit times (<= 0: the default, about 1-2
- * seconds); a wait that runs out ends its block and latches LB_E_TIMEOUT,
- * which lb_batch_sync and lb_batch_heat_flux report (the instances are then
- * only partly advanced and must be reset). */
+ * block), and the blocks wait for one another between steps. Results are
+ * bit-identical to stepping each instance alone. Each of those waits polls a
+ * device counter at most wait_limit times (<= 0: the default, some seconds);
+ * a wait that runs out ends its block and latches LB_E_TIMEOUT, which
+ * lb_batch_sync and lb_batch_heat_flux report (the instances are then only
+ * partly advanced and must be reset). */
 int lb_batch_set_persistent(lb_batch* b, int tiles_per_block, long long wait_limit);
 
 /* Per-instance heat-flux statistics into arrays of n entries (any may be

@@ -12,8 +12,9 @@ namespace lbgpu {
 
 namespace {
 
-struct MarchForm {
-    static constexpr int threads = MARCH_T, min_blocks = 4;
+template <int MINB>
+struct MarchFormT {
+    static constexpr int threads = MARCH_T, min_blocks = MINB;
     static constexpr int smem = MarchSmem::total * (int)sizeof(float2);
     template <bool REC, bool CG, bool OUT, bool QF>
     static __device__ __forceinline__ void body(const StepParams& P, const StepParams& C, int block, int fold,
@@ -21,6 +22,12 @@ struct MarchForm {
         march_body<REC, CG, OUT, QF>(P, C, block, fold, R);
     }
 };
+
+using MarchForm = MarchFormT<4>;
+// 168 registers: no faster at full load (310 us on 4096^2 against 302), but
+// half as many blocks again fit, so a batch's tiles come in finer steps of
+// one wave (36 domains of 600 x 150: 85 us per step against 101).
+using March6 = MarchFormT<6>;
 
 template <int NW, int K>
 struct TileForm {

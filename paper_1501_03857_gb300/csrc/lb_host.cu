@@ -307,20 +307,23 @@ StepParams step_params(const lb_handle* h, const StepParams& base, int cur) {
 inline int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
 
 // Column strips and most rows of one pass of a form's block.
-inline int form_strips(int form, int Lx) { return ceil_div(Lx, form == FORM_MARCH ? 2 * TILE_COLS : TILE_COLS); }
+inline bool form_marches(int form) { return form == FORM_MARCH || form == FORM_MARCH6; }
+inline int form_strips(int form, int Lx) { return ceil_div(Lx, form_marches(form) ? 2 * TILE_COLS : TILE_COLS); }
 inline int form_rows(int form) { return form == FORM_TILE16 ? TILE16_ROWS : form == FORM_TILE24 ? TILE24_ROWS : INT32_MAX; }
 
 // About how long a step of `blocks` blocks of seg_rows rows takes, in us, on
 // nsm SMs that hold occ blocks each: the forms' measured times. A tile takes
 // the same time whatever its SM's neighbours do, wave after wave; a marching
 // block takes its rows plus the pipeline's ten, two per iteration, and its
-// iterations hardly lengthen until the SM's four blocks are there.
+// iterations lengthen with the blocks on the fullest SM (the six-block form's
+// more, being the same work in fewer registers).
 double form_us(int form, long long blocks, int seg_rows, int nsm, int occ) {
     const long long waves = ceil_div(blocks, (long long)nsm * occ);
     if (form == FORM_TILE16) return 0.5 + 4.1 * waves * ceil_div(seg_rows, TILE16_ROWS);
     if (form == FORM_TILE24) return 0.8 + 5.7 * waves * ceil_div(seg_rows, TILE24_ROWS);
-    const double per_sm = std::min((double)occ, (double)blocks / nsm);
-    return 1.0 + waves * ceil_div(seg_rows + 2 * HALO, 2) * (1.75 + 0.13 * per_sm);
+    const int per_sm = (int)std::min<long long>(occ, ceil_div(blocks, nsm));
+    const double iter = form == FORM_MARCH ? 1.75 + 0.13 * per_sm : 1.85 + 0.26 * per_sm;
+    return 1.0 + waves * ceil_div(seg_rows + 2 * HALO, 2) * iter;
 }
 
 // The launch shape of one form for this grid (seg_rows 0: automatic): a tile
@@ -1007,8 +1010,7 @@ struct lb_batch {
     std::vector<lb_handle*> inst;
     std::vector<size_t> ws_off;  // workspace offset of each instance
     StepParams* table;           // device [2][n]: parameters by step parity
-    int* block_off;              // device [n + 1]: first block of each instance
-    std::vector<int> h_off;
+    std::vector<int> h_off;      // [n + 1]: first block (tile) of each instance
     std::vector<StepParams> h_table;
     int block_x, seg_req;        // launch shape asked for (seg_req 0: automatic)
     int form, threads;           // the form in use and its block size
@@ -1028,10 +1030,9 @@ struct lb_batch {
     int max_tiles;               // capacity of the tile arrays
     int2* d_tiles;               // device [max_tiles]: (instance, block index)
     int* d_tile_off;             // device [max_tiles + 1]: first tile of each block
-    int* d_ntiles;               // device [n]
-    unsigned* d_arrive;          // device [n]
+    unsigned* d_arrive;          // device: the barrier's counters
     std::vector<int2> h_tiles;
-    std::vector<int> h_tile_off, h_ntiles;
+    std::vector<int> h_tile_off;
     int pgrid;                   // blocks of the persistent launch
     cudaGraphExec_t pgraph;      // PERSIST_STEPS steps in one launch
     Acc* rec;                    // pinned [n]: the instances' records as last read
@@ -1041,7 +1042,7 @@ namespace {
 
 constexpr int GRAPH_STEPS = 32;  // steps per captured graph (even: parity returns)
 constexpr int PERSIST_STEPS = 32;  // steps per persistent launch in the captured graph (even)
-constexpr unsigned long long PERSIST_WAIT_DEFAULT = 1ull << 24;  // polls (64 ns sleeps): about 1-2 s
+constexpr unsigned long long PERSIST_WAIT_DEFAULT = 1ull << 23;  // polls (32 ns sleeps and a trip to L2): some seconds
 
 size_t batch_tail_offset(const lb_batch_desc* d, int n, std::vector<size_t>* offs) {
     size_t off = 0;
@@ -1062,19 +1063,17 @@ long long batch_max_tiles(const lb_batch_desc* d, int n) {
 
 // Byte offsets of the batch's device arrays after the instances' workspaces.
 struct BatchTail {
-    size_t table, block_off, tiles, tile_off, ntiles, arrive, total;
+    size_t table, tiles, tile_off, arrive, total;
 };
 
 BatchTail batch_tail(const lb_batch_desc* d, int n) {
     BatchTail T;
     const long long mt = batch_max_tiles(d, n);
     T.table = align256(batch_tail_offset(d, n, nullptr));
-    T.block_off = align256(T.table + 2 * n * sizeof(StepParams));
-    T.tiles = align256(T.block_off + (n + 1) * sizeof(int));
+    T.tiles = align256(T.table + 2 * n * sizeof(StepParams));
     T.tile_off = align256(T.tiles + (size_t)mt * sizeof(int2));
-    T.ntiles = align256(T.tile_off + (size_t)(mt + 1) * sizeof(int));
-    T.arrive = align256(T.ntiles + n * sizeof(int));
-    T.total = align256(T.arrive + n * sizeof(unsigned));
+    T.arrive = align256(T.tile_off + (size_t)(mt + 1) * sizeof(int));
+    T.total = align256(T.arrive + persist_arrive_bytes);
     return T;
 }
 
@@ -1136,8 +1135,8 @@ int batch_layout(lb_batch* b) {
     batch_constants(b);
     const int waves = std::max(1, b->tpb);
     double best = 0;
-    for (int form : {FORM_MARCH, FORM_TILE24}) {
-        if (form != FORM_MARCH && b->block_x == 64) continue;
+    for (int form : {FORM_MARCH, FORM_MARCH6, FORM_TILE24}) {
+        if (form == FORM_TILE24 && b->block_x == 64) continue;
         int threads = 0, o = 0;
         LB_CUDA(batch_occupancy(form, b->kshared, b->tpb > 0, &threads, &o), "occupancy");
         if (o < 1) return fail(LB_E_INVAL, "the batched step's block of %d threads does not fit on an SM", threads);
@@ -1169,27 +1168,29 @@ int batch_layout(lb_batch* b) {
         cudaGraphExecDestroy(b->pgraph);
         b->pgraph = nullptr;
     }
-    LB_CUDA(cudaMemcpyAsync(b->block_off, b->h_off.data(), (n + 1) * sizeof(int), cudaMemcpyHostToDevice, b->st),
-            "batch offsets upload");
+    const int ntile = b->nblocks;
+    if (ntile > b->max_tiles) return fail(LB_E_INVAL, "batch has %d tiles, more than the %d provided for", ntile, b->max_tiles);
+    std::vector<int2> tiles(ntile);  // (instance, block index within it)
+    for (int i = 0; i < n; ++i)
+        for (int t = b->h_off[i]; t < b->h_off[i + 1]; ++t) tiles[t] = make_int2(i, t - b->h_off[i]);
+    if (b->tpb == 0) {
+        b->h_tiles = tiles;
+        LB_CUDA(cudaMemcpyAsync(b->d_tiles, b->h_tiles.data(), ntile * sizeof(int2), cudaMemcpyHostToDevice, b->st),
+                "tiles upload");
+    }
     if (b->tpb > 0) {
         // Deal the tiles out to a grid of at most one wave, longest first to
         // the least loaded block (a tile costs its rows plus the pipeline's
         // 10 rows of halo); each block then takes its tiles in (instance,
         // tile) order, the same order on every block.
-        const int ntile = b->nblocks;
-        if (ntile > b->max_tiles) return fail(LB_E_INVAL, "batch has %d tiles, more than the %d provided for", ntile, b->max_tiles);
         const int G = std::min(ntile, nsm * occ);
         std::vector<std::pair<int, int>> order;  // (cost, tile)
-        std::vector<int2> tiles(ntile);
-        b->h_ntiles.assign(n, 0);
         for (int i = 0; i < n; ++i) {
             lb_handle* h = b->inst[i];
             const int nt = b->h_off[i + 1] - b->h_off[i];
-            b->h_ntiles[i] = nt;
             for (int k = 0; k < nt; ++k) {
                 const int seg = k / h->launch.nstrips;
                 const int rows = std::min(h->launch.seg_rows, h->grid.Ly - seg * h->launch.seg_rows);
-                tiles[b->h_off[i] + k] = make_int2(i, k);
                 order.push_back({rows + 2 * HALO, b->h_off[i] + k});
             }
         }
@@ -1227,8 +1228,6 @@ int batch_layout(lb_batch* b) {
         LB_CUDA(cudaMemcpyAsync(b->d_tile_off, b->h_tile_off.data(), (G + 1) * sizeof(int), cudaMemcpyHostToDevice,
                                 b->st),
                 "tile offsets upload");
-        LB_CUDA(cudaMemcpyAsync(b->d_ntiles, b->h_ntiles.data(), n * sizeof(int), cudaMemcpyHostToDevice, b->st),
-                "tile counts upload");
     }
     b->dirty = true;
     return LB_OK;
@@ -1254,7 +1253,7 @@ int batch_upload(lb_batch* b) {
 
 int batch_launch_one(lb_batch* b, cudaStream_t s, int parity, bool fold) {
     const int n = (int)b->inst.size();
-    LB_CUDA(batch_launch(b->form, b->table + parity * n, b->block_off, n, b->nblocks,
+    LB_CUDA(batch_launch(b->form, b->table + parity * n, b->d_tiles, b->nblocks,
                          b->kshared ? &b->kconst : nullptr, fold, s),
             "batch step launch");
     return LB_OK;
@@ -1267,19 +1266,18 @@ int batch_fold_last(lb_batch* b, cudaStream_t s, int parity) {
     return LB_OK;
 }
 
-// One persistent launch of `nsteps` steps (the arrival counters zeroed first).
+// One persistent launch of `nsteps` steps (the barrier zeroed first).
 int persist_launch_one(lb_batch* b, cudaStream_t s, int nsteps) {
     const int n = (int)b->inst.size();
     PersistArgs A;
     A.table = b->table;
     A.tiles = b->d_tiles;
     A.tile_off = b->d_tile_off;
-    A.ntiles = b->d_ntiles;
     A.arrive = b->d_arrive;
     A.n = n;
     A.nsteps = nsteps;
     A.wait_limit = b->wait_limit;
-    LB_CUDA(cudaMemsetAsync(b->d_arrive, 0, n * sizeof(unsigned), s), "clear arrival counters");
+    LB_CUDA(cudaMemsetAsync(b->d_arrive, 0, persist_arrive_bytes, s), "clear barrier");
     LB_CUDA(persist_launch(b->form, b->kshared ? &b->kconst : nullptr, A, b->pgrid, s), "persistent batch launch");
     return batch_fold_last(b, s, nsteps & 1);
 }
@@ -1362,7 +1360,6 @@ int lb_batch_init(lb_batch** out, const lb_batch_desc* d, int n, void* dev_works
     if (((uintptr_t)dev_workspace) & 255) return fail(LB_E_INVAL, "workspace must be 256-byte aligned");
     lb_batch* b = new lb_batch();
     b->table = nullptr;
-    b->block_off = nullptr;
     b->graph = nullptr;
     b->st = (cudaStream_t)stream;
     b->gs = nullptr;
@@ -1376,7 +1373,7 @@ int lb_batch_init(lb_batch** out, const lb_batch_desc* d, int n, void* dev_works
     b->pgrid = 0;
     b->pgraph = nullptr;
     b->d_tiles = nullptr;
-    b->d_tile_off = b->d_ntiles = nullptr;
+    b->d_tile_off = nullptr;
     b->d_arrive = nullptr;
     b->rec = nullptr;
     char* ws = (char*)dev_workspace;
@@ -1395,10 +1392,8 @@ int lb_batch_init(lb_batch** out, const lb_batch_desc* d, int n, void* dev_works
     const BatchTail T = batch_tail(d, n);
     (void)tail;
     b->table = (StepParams*)(ws + T.table);
-    b->block_off = (int*)(ws + T.block_off);
     b->d_tiles = (int2*)(ws + T.tiles);
     b->d_tile_off = (int*)(ws + T.tile_off);
-    b->d_ntiles = (int*)(ws + T.ntiles);
     b->d_arrive = (unsigned*)(ws + T.arrive);
     b->max_tiles = (int)std::min<long long>(batch_max_tiles(d, n), INT32_MAX);
     cudaError_t e = batch_prepare();

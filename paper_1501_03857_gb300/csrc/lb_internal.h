@@ -8,8 +8,9 @@
 
 namespace lbgpu {
 
-// Forms of the fused step (lb_march.cuh, lb_tile.cuh).
-enum Form { FORM_MARCH = 0, FORM_TILE16 = 1, FORM_TILE24 = 2, FORM_COUNT = 3 };
+// Forms of the fused step (lb_march.cuh, lb_tile.cuh); the last, marching with
+// six blocks per SM instead of four, for batches only.
+enum Form { FORM_MARCH = 0, FORM_TILE16 = 1, FORM_TILE24 = 2, FORM_COUNT = 3, FORM_MARCH6 = 3 };
 
 // Launch shape of the fused step: nstrips x nseg blocks of seg_rows rows
 // each; block_x threads per block (the form's).
@@ -44,31 +45,31 @@ cudaError_t launch_recompute(const StepParams& P, const RecomputeOut& R, bool ou
                              const Launch& L, cudaStream_t st);
 
 // The same step over a table of independent instances in one launch (the
-// marching form and the 24-row tiles); instance i owns blocks
-// [block_off[i], block_off[i+1]).
+// marching forms and the 24-row tiles): block g computes tiles[g] (instance,
+// block index within the instance).
 cudaError_t batch_prepare();
 cudaError_t batch_occupancy(int form, bool shared_k, bool persistent, int* threads, int* blocks_per_sm);
 // K non-null: every instance shares the model constants in *K and the kernel
 // reads them from its parameters. fold as in launch_step, batch_fold as
 // launch_fold (given the table of the step that would follow).
-cudaError_t batch_launch(int form, const StepParams* table, const int* block_off, int n, int nblocks,
-                         const StepParams* K, bool fold, cudaStream_t st);
+cudaError_t batch_launch(int form, const StepParams* table, const int2* tiles, int nblocks, const StepParams* K,
+                         bool fold, cudaStream_t st);
 cudaError_t batch_fold(const StepParams* table, int n, cudaStream_t st);
 
 // The persistent batch (lb_batch_persist in lb_step_batch.cu): one cooperative
 // launch of a fixed grid advances every instance by nsteps steps; block g
 // takes tiles tile_off[g] .. tile_off[g+1]-1 (instance, block index within
-// the instance) every step, after all tiles of the instance finished the
-// previous step (arrive[i] counts finished tiles of instance i since the
-// launch began and must be zero at launch). A wait gives up after
-// wait_limit polls, sets ERR_TIMEOUT in the instance's fault flags and ends
+// the instance) every step, with a barrier of all blocks between steps
+// (arrive: persist_arrive_bytes, zero at launch). A wait gives up after
+// wait_limit polls, sets ERR_TIMEOUT in an instance's fault flags and ends
 // the block.
+constexpr int PERSIST_SUB = 32, PERSIST_PAD = 8;  // first-level counters, a sector each
+constexpr size_t persist_arrive_bytes = sizeof(unsigned) * (PERSIST_SUB + 1) * PERSIST_PAD;
 struct PersistArgs {
     const StepParams* table;  // [2][n], by step parity
     const int2* tiles;
     const int* tile_off;
-    const int* ntiles;        // [n] tiles per instance
-    unsigned* arrive;         // [n]
+    unsigned* arrive;
     int n, nsteps;
     unsigned long long wait_limit;
 };

@@ -1,50 +1,40 @@
 // Many independent simulations in one launch (the boiling-curve batch): one
 // launch per step, or one cooperative launch for a run of steps. The
-// marching form and the taller tiles of the fused step (lb_march.cuh,
-// lb_tile.cuh).
+// marching form at four and at six blocks per SM and the taller tiles of the
+// fused step (lb_march.cuh, lb_tile.cuh).
 #include "lb_forms.cuh"
 
 namespace lbgpu {
 
 namespace {
 
-// The blocks of instance i are [block_off[i], block_off[i+1]); each block copies its instance's parameter record to shared memory (sP) and returns the
-// block's index within its instance.
+// Copy an instance's parameter record to shared memory; the block's threads
+// need a barrier before they use it.
 template <int BD>
-__device__ __forceinline__ int batch_instance(const StepParams* __restrict__ table, const int* __restrict__ block_off,
-                                              int n, StepParams& sP) {
-    __shared__ int s_inst;
-    if (threadIdx.x == 0) {
-        int lo = 0, hi = n - 1;  // largest i with block_off[i] <= blockIdx.x
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (block_off[mid] <= (int)blockIdx.x) lo = mid;
-            else hi = mid - 1;
-        }
-        s_inst = lo;
-    }
-    __syncthreads();
-    const int inst = s_inst;
+__device__ __forceinline__ void copy_params(const StepParams* __restrict__ src, StepParams& dst) {
     constexpr int NW = (int)(sizeof(StepParams) / sizeof(int));
     static_assert(sizeof(StepParams) % sizeof(int) == 0, "StepParams is copied as ints");
     for (int k = threadIdx.x; k < NW; k += BD)
-        reinterpret_cast<int*>(&sP)[k] = __ldg(reinterpret_cast<const int*>(table + inst) + k);
-    __syncthreads();
-    return (int)blockIdx.x - block_off[inst];
+        reinterpret_cast<int*>(&dst)[k] = __ldg(reinterpret_cast<const int*>(src) + k);
 }
 
-// The batch with every model constant from the instance's record (SK false),
-// or with the constants that all instances share in K, in the parameter bank
-// (the table then supplies each instance's buffers, sizes, launch shape,
-// wettability and rho_ave).
+// One step of the batch: block g computes tiles[g] (instance, block index
+// within it), with every model constant from the instance's record (SK
+// false), or with the constants that all instances share in K, in the
+// parameter bank (the table then supplies each instance's buffers, sizes,
+// launch shape, wettability and rho_ave). The record is fetched before the
+// block waits for the step before it: no kernel writes the table, and a copy
+// into it is complete before the launch that follows it starts.
 template <class F, bool SK>
 __global__ void __launch_bounds__(F::threads, F::min_blocks)
-    lb_step_batch(const StepParams K, const StepParams* __restrict__ table, const int* __restrict__ block_off, const int n,
-                  const int fold) {
+    lb_step_batch(const StepParams K, const StepParams* __restrict__ table, const int2* __restrict__ tiles, const int fold) {
     __shared__ StepParams sP;
-    grid_start();
-    const int b = batch_instance<F::threads>(table, block_off, n, sP);
-    F::template body<false, false, true, true>(sP, SK ? K : sP, b, fold, nullptr);
+    asm volatile("griddepcontrol.launch_dependents;");
+    const int2 tl = __ldg(tiles + blockIdx.x);
+    copy_params<F::threads>(table + tl.x, sP);
+    __syncthreads();
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    F::template body<false, false, true, true>(sP, SK ? K : sP, tl.y, fold, nullptr);
 }
 
 // q(t) of every instance's last step of a call: one warp per instance, from
@@ -57,127 +47,82 @@ __global__ void __launch_bounds__(32) lb_batch_fold(const StepParams* __restrict
 // ---------------------------------------------------------------------------
 // The persistent batch: one launch advances every instance by `nsteps` steps.
 //
-// The instances' tiles (a pair of column strips x a segment of rows, the
-// unit one block of the per-step kernel computes) are dealt out to a fixed,
-// co-resident grid (a cooperative launch); block g takes tiles
-// tile_off[g] .. tile_off[g+1]-1 in that order, step after step. A tile may
-// start step k once every tile of its instance has finished step k-1:
-// its pulled rows and the strips beside it are then complete (read after
-// write), and no tile of the instance still reads the buffer step k writes
-// (write after read). arrive[i] counts the tiles of instance i that have
-// finished a step since the launch began (zeroed before each launch), so
-// the wait is arrive[i] >= k * ntiles[i]. The wait spins at most
-// `wait_limit` polls (with a short sleep between them); a block that gives
-// up sets ERR_TIMEOUT in its instance's fault flags and leaves the kernel,
-// which lets every block waiting on it give up in turn, so the launch always
-// ends. The step's input state is read with plain loads, which after the
-// acquiring wait and the barrier see the other SMs' writes (the read-only
-// path could serve copies cached before them), and every tile runs the same
-// step body as the per-step kernel, so results are bit-identical to it.
+// The instances' tiles (what one block of the per-step kernel computes) are
+// dealt out to a fixed, co-resident grid (a cooperative launch); block g takes
+// tiles tile_off[g] .. tile_off[g+1]-1 in that order, step after step, and the
+// blocks meet at a barrier between steps: a tile's pulled rows and the strips
+// beside it are then complete (read after write), and no tile still reads the
+// buffer the step writes (write after read). The barrier counts in two levels
+// (arrive: PERSIST_SUB counters, the last arrival at each adds to a root; all
+// zero at launch). A wait polls the root at most `wait_limit` times; a block
+// that gives up sets ERR_TIMEOUT in its first instance's fault flags and
+// leaves the kernel, which lets every block waiting on it give up in turn, so
+// the launch always ends. The step's input state is read with plain loads,
+// which after the acquiring fence and the block's barrier see the other SMs'
+// writes (the read-only path could serve copies cached before them), and every
+// tile runs the same step as the per-step kernel, so results are bit-identical
+// to it.
+//
+// Waiting only for the tile's own instance, as this kernel did before, lets
+// the instances drift apart, and blocks at different stages of their march
+// evict each other's instructions (36 domains of 600 x 150: no-instruction
+// stalls 1.8 cycles per issue against 0.4 per-step, 99 us per step against 92
+// with the common barrier; 48 uneven domains 151 against 144).
 // ---------------------------------------------------------------------------
-
-// Poll *p until it reaches `target`, at most `limit` times; true if reached.
-__device__ __forceinline__ bool wait_at_least(const unsigned* p, unsigned target, unsigned long long limit) {
-    for (unsigned long long it = 0;; ++it) {
-        unsigned v;
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-        if (v >= target) return true;
-        if (it >= limit) return false;
-        __nanosleep(64);
-    }
-}
-
-// The most tiles one block of the persistent batch schedules by readiness
-// (more than this many are taken in order).
-constexpr int PERSIST_MAX_TILES = 64;
 
 template <class F, bool SK>
 __global__ void __launch_bounds__(F::threads, F::min_blocks) lb_batch_persist(const StepParams K, const PersistArgs A) {
     constexpr int BD = F::threads;
     __shared__ StepParams sP;
-    __shared__ int s_next[PERSIST_MAX_TILES];  // next step of each of the block's tiles
-    __shared__ int s_pick;
-    const int t0 = A.tile_off[blockIdx.x], t1 = A.tile_off[blockIdx.x + 1];
-    const int m = t1 - t0;
-    const bool by_ready = m <= PERSIST_MAX_TILES;
-    for (int j = threadIdx.x; j < PERSIST_MAX_TILES; j += BD) s_next[j] = 0;
-    __syncthreads();
-    // whether tile j may run its next step: every tile of its instance has
-    // finished the previous one
-    auto ready = [&](int j, int k) {
-        const int inst = A.tiles[t0 + j].x;
-        unsigned v;
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(A.arrive + inst) : "memory");
-        return k == 0 || v >= (unsigned)k * (unsigned)A.ntiles[inst];
-    };
-    int last = m - 1, done_in_order = 0;
-    for (;;) {
-        // thread 0 picks the next tile: with few tiles per block the first
-        // ready one after the last tile run (round robin), so a block never
-        // idles while one of its tiles can go on; otherwise the tiles in
-        // order, step after step. -2: all done; -3: a wait ran out.
-        if (threadIdx.x == 0) {
-            int pick = -2;
-            if (by_ready) {
-                unsigned long long polls = 0;
-                for (;;) {
-                    bool left = false;
-                    pick = -1;
-                    for (int d = 1; d <= m; ++d) {
-                        const int j = (last + d) % m;
-                        if (s_next[j] >= A.nsteps) continue;
-                        left = true;
-                        if (ready(j, s_next[j])) {
-                            pick = j;
-                            break;
-                        }
-                    }
-                    if (!left) {
-                        pick = -2;
-                        break;
-                    }
-                    if (pick >= 0) break;
-                    if (polls++ >= A.wait_limit) {
-                        pick = -3;
-                        break;
-                    }
-                    __nanosleep(64);
+    __shared__ bool s_go;
+    const int t0 = A.tile_off[blockIdx.x], m = A.tile_off[blockIdx.x + 1] - t0;
+    const unsigned G = gridDim.x, nsub = min(G, (unsigned)PERSIST_SUB), sub = blockIdx.x % nsub;
+    const unsigned size = (G - sub + nsub - 1) / nsub;  // blocks that count at this block's counter
+    unsigned* const root = A.arrive + PERSIST_SUB * PERSIST_PAD;
+    for (int k = 0; k < A.nsteps; ++k) {
+        if (k > 0) {
+            if (threadIdx.x == 0) {
+                bool go = false;
+                for (unsigned long long it = 0;; ++it) {
+                    unsigned v;
+                    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(root) : "memory");
+                    go = v >= (unsigned)k * nsub;
+                    if (go || it >= A.wait_limit) break;
+                    __nanosleep(32);
                 }
-            } else if (done_in_order < m * A.nsteps) {
-                const int j = done_in_order % m, k = done_in_order / m;
-                pick = wait_at_least(A.arrive + A.tiles[t0 + j].x, (unsigned)k * (unsigned)A.ntiles[A.tiles[t0 + j].x],
-                                     k == 0 ? 0ull : A.wait_limit) || k == 0 ? j : -3;
-                if (pick >= 0) s_next[0] = k;  // the step to run
+                if (!go) atomicOr(&A.table[A.tiles[t0].x].acc->err, ERR_TIMEOUT);
+                asm volatile("fence.acq_rel.gpu;" ::: "memory");
+                s_go = go;
             }
-            if (pick == -3) {  // latch the timeout on an unfinished tile's instance
-                for (int j = 0; j < m; ++j)
-                    if (!by_ready || s_next[j] < A.nsteps) {
-                        atomicOr(&A.table[A.tiles[t0 + j].x].acc->err, ERR_TIMEOUT);
-                        break;
-                    }
-            }
-            s_pick = pick;
+            __syncthreads();
+            if (!s_go) return;
         }
-        __syncthreads();
-        const int pick = s_pick;
-        if (pick < 0) return;  // all done, or given up
-        const int k = by_ready ? s_next[pick] : s_next[0];
-        const int2 tl = A.tiles[t0 + pick];
-        const StepParams* src = A.table + (k & 1) * A.n + tl.x;
-        constexpr int NW = (int)(sizeof(StepParams) / sizeof(int));
-        for (int w = threadIdx.x; w < NW; w += BD)
-            reinterpret_cast<int*>(&sP)[w] = __ldg(reinterpret_cast<const int*>(src) + w);
-        __syncthreads();
-        F::template body<false, true, true, true>(sP, SK ? K : sP, tl.y, k > 0, nullptr);
-        __syncthreads();
+        for (int j = 0; j < m; ++j) {
+            const int2 tl = A.tiles[t0 + j];
+            if (m > 1 || k == 0) {
+                copy_params<BD>(A.table + (k & 1) * A.n + tl.x, sP);
+                __syncthreads();
+            }
+            F::template body<false, true, true, true>(sP, SK ? K : sP, tl.y, k > 0, nullptr);
+            __syncthreads();
+        }
         if (threadIdx.x == 0) {
             __threadfence();
-            atomicAdd(A.arrive + tl.x, 1u);
-            if (by_ready) ++s_next[pick];
-            else ++done_in_order;
-            last = pick;
+            if (atomicAdd(A.arrive + sub * PERSIST_PAD, 1u) == (unsigned)(k + 1) * size - 1u) {
+                __threadfence();
+                atomicAdd(root, 1u);
+            }
+            if (m == 1) {  // the other parity's record is this one with its buffers exchanged
+                const StepParams P = sP;
+                sP.f_in = P.f_out;
+                sP.f_out = const_cast<float*>(P.f_in);
+                sP.th_in = P.th_out;
+                sP.th_out = const_cast<float*>(P.th_in);
+                sP.qpart = const_cast<double*>(P.qprev);
+                sP.qprev = P.qpart;
+            }
         }
-        __syncthreads();
+        // (the next step's first barrier, at the wait above, orders sP)
     }
 }
 
@@ -211,6 +156,7 @@ struct BatchForm {
 template <class F>
 auto with_batch_form(int form, F f) {
     if (form == FORM_TILE24) return f(Tile24{});
+    if (form == FORM_MARCH6) return f(March6{});
     return f(MarchForm{});
 }
 
@@ -218,6 +164,7 @@ auto with_batch_form(int form, F f) {
 
 cudaError_t batch_prepare() {
     cudaError_t e = BatchForm<MarchForm>::prepare();
+    if (e == cudaSuccess) e = BatchForm<March6>::prepare();
     return e == cudaSuccess ? BatchForm<Tile24>::prepare() : e;
 }
 
@@ -231,13 +178,13 @@ cudaError_t batch_occupancy(int form, bool shared_k, bool persistent, int* threa
     });
 }
 
-cudaError_t batch_launch(int form, const StepParams* table, const int* block_off, int n, int nblocks,
-                         const StepParams* K, bool fold, cudaStream_t st) {
+cudaError_t batch_launch(int form, const StepParams* table, const int2* tiles, int nblocks, const StepParams* K,
+                         bool fold, cudaStream_t st) {
     const StepParams k0 = K ? *K : StepParams{};
     return with_batch_form(form, [&](auto f) {
         using F = decltype(f);
         auto kernel = K ? lb_step_batch<F, true> : lb_step_batch<F, false>;
-        return launch_after(kernel, nblocks, F::threads, F::smem, st, k0, table, block_off, n, (int)fold);
+        return launch_after(kernel, nblocks, F::threads, F::smem, st, k0, table, tiles, (int)fold);
     });
 }
 
