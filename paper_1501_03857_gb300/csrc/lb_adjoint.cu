@@ -29,7 +29,7 @@
 // y or the outflow top, with or without the ghost layer (the host checks).
 #include <algorithm>
 
-#include "lb_internal.h"
+#include "lb_common.cuh"
 
 namespace lbgpu {
 
@@ -158,6 +158,8 @@ __device__ __forceinline__ void rev_coef_vals(const StepParams& P, const AdjFiel
     LB_ST(A.lvx, i, P.plane, -lax);
     LB_ST(A.lvy, i, P.plane, -lay);
 }
+
+#include "lb_rev_tile.cuh"
 
 // ---- the four RK stages transposed in one column-marching launch ------------
 //
@@ -410,6 +412,7 @@ __global__ void __launch_bounds__(RT_BD) rev_thermal_fused(const StepParams P, A
     for (; L <= hi + RT_HALO; ++L) iter(L, std::false_type{});
 }
 
+constexpr int RV_NW = 12, RV_K = 2, RV_SMEM = RevShape2<RV_NW, RV_K>::slots * (int)sizeof(float2);
 constexpr size_t rt_smem_bytes() { return sizeof(float) * (size_t)RT_SMN; }
 
 // ---- collision, forces, psi and the pull transposed in one column-marching launch
@@ -945,12 +948,24 @@ cudaError_t adjoint_reverse_step(const StepParams& P, const RecomputeOut& R, voi
         if (r.e == cudaSuccess)
             r.e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r.occ_t, rev_thermal_fused, RT_BD, rt_smem_bytes());
         if (r.e == cudaSuccess) r.e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r.occ_f, rev_flow_fused, RF_BD, 0);
+        if (r.e == cudaSuccess) r.e = allow_smem((const void*)rev_tile<RV_NW, RV_K>, RV_SMEM);
         r.occ_t = std::max(r.occ_t, 1);
         r.occ_f = std::max(r.occ_f, 1);
         return r;
     }();
     if (RS.e != cudaSuccess) return RS.e;
     const int nsm = RS.nsm, occ_t = RS.occ_t, occ_f = RS.occ_f;
+    const int tiles = (P.Lx + RV_COLS - 1) / RV_COLS * rev_tiles<RevShape2<RV_NW, RV_K>>(P.Ly);
+    // the tiles while they come to three waves at most (one block per SM, 13
+    // us a wave): the marching kernels take 26 us at the least and overtake
+    // at four waves (512^2: 62 us against 66 with the forward step; 517 x
+    // 1003, six waves: 114 against 93)
+    if (tiles <= 3 * nsm) {
+        StepParams Q = P;  // the pull reads the state through the parameters
+        Q.f_in = fstar;
+        Q.th_in = theta;
+        return launch_after(rev_tile<RV_NW, RV_K>, tiles, RV_NW * 32, RV_SMEM, st, Q, A, lq);
+    }
     // (a floor of 4 rows per segment: on small domains more, shorter marches
     // beat fewer long ones despite the halo rows; measured cost of the 256^2,
     // 2000-step adjoint against its forward steps: 2.78x at 4, 2.90x at 1,

@@ -3,8 +3,6 @@
 // recompute mode; lb_step_batch.cu: batches).
 #pragma once
 
-#include <algorithm>
-
 #include "lb_march.cuh"
 #include "lb_tile.cuh"
 
@@ -44,36 +42,6 @@ using Tile24 = TileForm<12, 2>;
 static_assert(TileShape<16, 1>::out == TILE16_ROWS && TileShape<12, 2>::out == TILE24_ROWS && TILE_OUT == TILE_COLS &&
                   MARCH_COLS == 2 * TILE_COLS,
               "the host's launch shapes use these");
-
-// Wait for the work this grid depends on. Every kernel of the step is
-// launched to start while its predecessor in the stream drains
-// (launch_after), so it waits here before it touches memory; the first
-// instruction lets its own successor do the same.
-__device__ __forceinline__ void grid_start() {
-    asm volatile("griddepcontrol.launch_dependents;");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-
-// Launch on `st` with the launch latency hidden behind the predecessor's last
-// blocks (programmatic dependent launch; 0.3 us of a 5 us step).
-template <class... A, class... B>
-cudaError_t launch_after(void (*kernel)(A...), int blocks, int threads, int smem, cudaStream_t st, B... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = (size_t)smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, A(args)...);
-}
-
-inline cudaError_t allow_smem(const void* kernel, int bytes) {
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-}
 
 // f(form) for the form a launch names (Form in lb_internal.h)
 template <class F>

@@ -28,9 +28,7 @@ namespace lbgpu {
 
 namespace {
 
-constexpr int TILE_W = 64;                   // columns a tile computes
 constexpr int TILE_OUT = TILE_W - 2 * HALO;  // columns it writes
-constexpr int TILE_ROW = 34;                 // float2 slots of a shared row
 
 template <int NW, int K>
 struct TileShape {
