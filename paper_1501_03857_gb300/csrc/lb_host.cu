@@ -1666,7 +1666,13 @@ int lb_adjoint(lb_handle* h, int nsteps, int ckpt_every, void* dev_scratch, size
                 "checkpoint copy");
         return LB_OK;
     };
-    if ((rc = save(sf(L.ckpt, 0), h->f[h->cur], h->t[h->cur]))) return rc;
+    // the states of an every-step window: the first and the last are the
+    // simulation's own two buffers (the sweep reads the first there, and the
+    // last is where the simulation goes on), the others checkpoints
+    const int c0 = h->cur;
+    auto state_f = [&](int n) { return n == 0 ? h->f[c0] : n == nsteps ? h->f[1 - c0] : sf(L.ckpt, n); };
+    auto state_t = [&](int n) { return n == 0 ? h->t[c0] : n == nsteps ? h->t[1 - c0] : sf(L.ckpt, n) + 9 * pl; };
+    if (C > 1 && (rc = save(sf(L.ckpt, 0), h->f[h->cur], h->t[h->cur]))) return rc;
     const size_t rec_stride = align256(sizeof(float) * kRecomputePlanes * pl);
     auto rec_at = [&](size_t k) {  // the k-th set of forward intermediates
         float* r = (float*)(s + L.rec + k * rec_stride);
@@ -1676,15 +1682,15 @@ int lb_adjoint(lb_handle* h, int nsteps, int ckpt_every, void* dev_scratch, size
     if (C == 1) {
         // every step stored: the forward pass runs the fused step in its
         // recompute mode with the step's output and q(t), writing state n+1
-        // into checkpoint n+1 and the step's intermediates into set n, so the
-        // reverse sweep replays nothing
+        // and the step's intermediates into set n, so the reverse sweep
+        // replays nothing
         for (int n = 0; n < nsteps; ++n) {
             StepParams P = step_params(h, base, n & 1);
             P.acc = acc;
-            P.f_in = sf(L.ckpt, n);
-            P.th_in = sf(L.ckpt, n) + 9 * pl;
-            P.f_out = sf(L.ckpt, n + 1);
-            P.th_out = sf(L.ckpt, n + 1) + 9 * pl;
+            P.f_in = state_f(n);
+            P.th_in = state_t(n);
+            P.f_out = state_f(n + 1);
+            P.th_out = state_t(n + 1);
             LB_CUDA(launch_recompute(P, rec_at(n), true, true, n > 0, h->launch, st), "adjoint forward step");
             if (h->probe.n > 0) {
                 ProbeArgs A = h->probe;
@@ -1698,15 +1704,7 @@ int lb_adjoint(lb_handle* h, int nsteps, int ckpt_every, void* dev_scratch, size
             P.acc = acc;
             if ((rc = fold_last(h, P, nsteps & 1, st))) return rc;
         }
-        // the simulation advances as with the plain steps: the last state
-        // into the current population and theta buffers (separate arrays of
-        // the workspace, not one 10-plane block like a checkpoint)
-        LB_CUDA(cudaMemcpyAsync(h->f[h->cur], sf(L.ckpt, nsteps), sizeof(float) * 9 * pl, cudaMemcpyDeviceToDevice,
-                                st),
-                "state copy");
-        LB_CUDA(cudaMemcpyAsync(h->t[h->cur], sf(L.ckpt, nsteps) + 9 * pl, sizeof(float) * pl,
-                                cudaMemcpyDeviceToDevice, st),
-                "state copy");
+        h->cur ^= 1;
         h->steps += nsteps;
     } else {
         StepParams P = base;
@@ -1782,8 +1780,7 @@ int lb_adjoint(lb_handle* h, int nsteps, int ckpt_every, void* dev_scratch, size
     auto sweep_all = [&](cudaStream_t q) -> int {
         int c = 0;
         for (int j = nsteps - 1; j >= 0; --j) {
-            const float* fs = sf(L.ckpt, j);
-            LB_CUDA(adjoint_reverse_step(RB, rec_at((size_t)j), work, fs, fs + 9 * pl, lam[c], lam[c] + 9 * pl,
+            LB_CUDA(adjoint_reverse_step(RB, rec_at((size_t)j), work, state_f(j), state_t(j), lam[c], lam[c] + 9 * pl,
                                          lam[c] + 10 * pl, lam[1 - c], lam[1 - c] + 9 * pl, lam[1 - c] + 10 * pl, lq, q),
                     "adjoint reverse step");
             c ^= 1;
@@ -1841,7 +1838,7 @@ int lb_adjoint(lb_handle* h, int nsteps, int ckpt_every, void* dev_scratch, size
     int cur = 0;
     if (C == 1) {
         cudaGraphExec_t g = nullptr;
-        if ((rc = graph_of(2, nsteps, 0, 0, rs, &g))) return rc;
+        if ((rc = graph_of(2, nsteps, c0, 0, rs, &g))) return rc;  // (the first state is buffer c0)
         LB_CUDA(cudaGraphLaunch(g, rs), "cudaGraphLaunch");
         cur = nsteps & 1;
     } else if ((rc = fill(kmax))) {
