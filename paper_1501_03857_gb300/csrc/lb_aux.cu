@@ -170,11 +170,13 @@ __global__ void __launch_bounds__(FIELD_T) fields_kernel(const StepParams P, flo
 // Rows of lx floats between arrays of row stride sp and dp, two arrays (the
 // populations' 9 Ly rows, theta's Ly) in one launch; V floats per access. A
 // warp takes 4 KB runs of a row, so that short rows do not leave lanes idle
-// for long and long ones keep many loads in flight.
+// for long and long ones keep many loads in flight. The fault flags go along
+// to host memory (a read of their own costs 4 us more).
 template <int V>
 __global__ void __launch_bounds__(256) copy_rows(const float* __restrict__ s0, float* __restrict__ d0, int n0,
                                                  const float* __restrict__ s1, float* __restrict__ d1, int n1, int lx,
-                                                 int sp, int dp) {
+                                                 int sp, int dp, const unsigned* err, unsigned* err_out) {
+    if (err_out && blockIdx.x == 0 && threadIdx.x == 0) *err_out = *err;
     using T = typename std::conditional<V == 4, float4, float>::type;
     constexpr int RUN = 1024;  // floats
     const int lane = threadIdx.x & 31;
@@ -282,7 +284,8 @@ cudaError_t launch_macro(const StepParams& P, float* scratch, float* rho, float*
 }
 
 cudaError_t launch_copy_state(const float* f_src, float* f_dst, const float* t_src, float* t_dst, int Lx, int Ly,
-                              int src_pitch, int dst_pitch, cudaStream_t st) {
+                              int src_pitch, int dst_pitch, const unsigned* err, unsigned* err_out,
+                              cudaStream_t st) {
     const int n0 = f_src ? 9 * Ly : 0, n1 = t_src ? Ly : 0;
     const uintptr_t all = (uintptr_t)f_src | (uintptr_t)f_dst | (uintptr_t)t_src | (uintptr_t)t_dst;
     const long long warps = (long long)(n0 + n1) * ((Lx + 1023) / 1024);
@@ -290,24 +293,25 @@ cudaError_t launch_copy_state(const float* f_src, float* f_dst, const float* t_s
     if (blocks == 0) return cudaSuccess;
     // (the pitch is a multiple of 32 floats: the other side's rows decide)
     if (all % 16 == 0 && Lx % 4 == 0)
-        copy_rows<4><<<blocks, 256, 0, st>>>(f_src, f_dst, n0, t_src, t_dst, n1, Lx, src_pitch, dst_pitch);
+        copy_rows<4><<<blocks, 256, 0, st>>>(f_src, f_dst, n0, t_src, t_dst, n1, Lx, src_pitch, dst_pitch, err, err_out);
     else
-        copy_rows<1><<<blocks, 256, 0, st>>>(f_src, f_dst, n0, t_src, t_dst, n1, Lx, src_pitch, dst_pitch);
+        copy_rows<1><<<blocks, 256, 0, st>>>(f_src, f_dst, n0, t_src, t_dst, n1, Lx, src_pitch, dst_pitch, err, err_out);
     return cudaGetLastError();
 }
 
-// The accumulator records of a batch's instances into out (host memory the
-// device can write), one thread each; reset clears the heat-flux sums.
-__global__ void collect_acc(const StepParams* __restrict__ table, int n, Acc* out, int reset) {
+// The accumulator records of a batch's instances (table) or of one simulation
+// (acc) into out (host memory the device can write), one thread each; reset
+// clears the heat-flux sums.
+__global__ void collect_acc(const StepParams* __restrict__ table, Acc* acc, int n, Acc* out, int reset) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    Acc* a = table[i].acc;
+    Acc* a = table ? table[i].acc : acc;
     out[i] = *a;
     if (reset) a->q_sum = a->q_sum2 = a->q_n = 0.0;
 }
 
-cudaError_t launch_collect(const StepParams* table, int n, Acc* out, bool reset, cudaStream_t st) {
-    collect_acc<<<(n + 63) / 64, 64, 0, st>>>(table, n, out, reset ? 1 : 0);
+cudaError_t launch_collect(const StepParams* table, Acc* acc, int n, Acc* out, bool reset, cudaStream_t st) {
+    collect_acc<<<(n + 63) / 64, 64, 0, st>>>(table, acc, n, out, reset ? 1 : 0);
     return cudaGetLastError();
 }
 

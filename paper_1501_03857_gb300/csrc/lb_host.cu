@@ -403,10 +403,10 @@ int report_device_errors(lb_handle* h, unsigned err) {
 }
 
 // The accumulator record into h->rec, after everything issued on the stream:
-// one copy to pinned memory and one wait (a read into pageable memory waits
-// once more).
-int read_acc(lb_handle* h) {
-    LB_CUDA(cudaMemcpyAsync(h->rec, h->acc, sizeof(Acc), cudaMemcpyDeviceToHost, h->st), "read accumulators");
+// one launch that writes pinned memory and one wait (a read into pageable
+// memory waits once more); reset clears the heat-flux sums.
+int read_acc(lb_handle* h, bool reset = false) {
+    LB_CUDA(launch_collect(nullptr, h->acc, 1, h->rec, reset, h->st), "read accumulators");
     LB_CUDA(cudaStreamSynchronize(h->st), "cudaStreamSynchronize");
     return LB_OK;
 }
@@ -727,14 +727,12 @@ static void flux_stats(const Acc& a, double* q_inst, double* q_mean, double* q_s
 
 int lb_heat_flux(lb_handle* h, double* q_inst, double* q_mean, double* q_std, int64_t* nsamples, int reset) {
     if (!h) return fail(LB_E_INVAL, "null handle");
-    // one read of the accumulator record, fault flags included; the reset
-    // follows it in stream order
-    int rc = read_acc(h);
+    // one read of the accumulator record, fault flags included
+    int rc = read_acc(h, reset != 0);
     if (rc) return rc;
     const Acc a = *h->rec;
     rc = report_device_errors(h, a.err);
     flux_stats(a, q_inst, q_mean, q_std, nsamples);
-    if (reset) LB_CUDA(cudaMemsetAsync(&h->acc->q_sum, 0, 3 * sizeof(double), h->st), "reset accumulators");
     return rc;
 }
 
@@ -766,11 +764,12 @@ int lb_get_state(lb_handle* h, float* fpost, float* theta, int on_device) {
     if (!h) return fail(LB_E_INVAL, "null handle");
     const int Lx = h->grid.Lx, Ly = h->grid.Ly, pitch = h->lay.pitch;
     const cudaMemcpyKind k = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-    if (on_device && (!fpost || on_this_device(fpost)) && (!theta || on_this_device(theta))) {
+    if (on_device && (fpost || theta) && (!fpost || on_this_device(fpost)) && (!theta || on_this_device(theta))) {
         LB_CUDA(launch_copy_state(fpost ? h->f[h->cur] : nullptr, fpost, theta ? h->t[h->cur] : nullptr, theta, Lx, Ly,
-                                  pitch, Lx, h->st),
+                                  pitch, Lx, &h->acc->err, &h->rec->err, h->st),
                 "state copy");
-        return check_device_errors(h);
+        LB_CUDA(cudaStreamSynchronize(h->st), "cudaStreamSynchronize");
+        return report_device_errors(h, h->rec->err);
     }
     if (fpost)
         LB_CUDA(cudaMemcpy2DAsync(fpost, Lx * sizeof(float), h->f[h->cur], pitch * sizeof(float), Lx * sizeof(float),
@@ -787,8 +786,9 @@ int lb_set_state(lb_handle* h, const float* fpost, const float* theta, int on_de
     if (!h) return fail(LB_E_INVAL, "null handle");
     const int Lx = h->grid.Lx, Ly = h->grid.Ly, pitch = h->lay.pitch;
     const cudaMemcpyKind k = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    if (on_device && (!fpost || on_this_device(fpost)) && (!theta || on_this_device(theta))) {
-        LB_CUDA(launch_copy_state(fpost, h->f[h->cur], theta, h->t[h->cur], Lx, Ly, Lx, pitch, h->st), "state copy");
+    if (on_device && (fpost || theta) && (!fpost || on_this_device(fpost)) && (!theta || on_this_device(theta))) {
+        LB_CUDA(launch_copy_state(fpost, h->f[h->cur], theta, h->t[h->cur], Lx, Ly, Lx, pitch, nullptr, nullptr, h->st),
+                "state copy");
         return LB_OK;
     }
     if (fpost)
@@ -1488,7 +1488,7 @@ int lb_batch_step(lb_batch* b, int nsteps) {
 static int batch_read(lb_batch* b, bool reset) {
     int rc = batch_upload(b);  // the table names the instances' records
     if (rc) return rc;
-    LB_CUDA(launch_collect(b->table, (int)b->inst.size(), b->rec, reset, b->st), "read accumulators");
+    LB_CUDA(launch_collect(b->table, nullptr, (int)b->inst.size(), b->rec, reset, b->st), "read accumulators");
     LB_CUDA(cudaStreamSynchronize(b->st), "cudaStreamSynchronize");
     int first = LB_OK;
     std::string msg;

@@ -109,13 +109,15 @@ cudaError_t adjoint_grads_finish(const StepParams& P, void* work, const float* l
                                  double* dGw_host, cudaStream_t st);
 
 // Populations (9 Ly rows) and theta (Ly rows) of Lx floats between device
-// arrays of different row strides; a null source is skipped.
+// arrays of different row strides; a null source is skipped (not both). With
+// err_out (pinned host memory) the flags *err go there.
 cudaError_t launch_copy_state(const float* f_src, float* f_dst, const float* t_src, float* t_dst, int Lx, int Ly,
-                              int src_pitch, int dst_pitch, cudaStream_t st);
+                              int src_pitch, int dst_pitch, const unsigned* err, unsigned* err_out, cudaStream_t st);
 
-// The accumulator records of a batch's instances (table[i].acc) into out, in
-// pinned host memory; reset clears the heat-flux sums after reading.
-cudaError_t launch_collect(const StepParams* table, int n, Acc* out, bool reset, cudaStream_t st);
+// The accumulator records of a batch's instances (table[i].acc), or with no
+// table the one at acc, into out, in pinned host memory; reset clears the
+// heat-flux sums after reading.
+cudaError_t launch_collect(const StepParams* table, Acc* acc, int n, Acc* out, bool reset, cudaStream_t st);
 
 // Record the message lb_last_error() returns on this thread.
 void set_last_error(const char* msg);
