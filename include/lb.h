@@ -173,8 +173,9 @@ int lb_info(lb_handle* h, int64_t* steps, int* block_x, int* seg_rows, int* nblo
 
 /* Override the launch shape of the fused step: block_x names its form (64:
  * blocks marching up column strips, for domains that fill the GPU; 128 and
- * 256: tiles of 24 and 16 computed rows, for smaller ones; 0: the one
- * expected to be fastest), seg_rows >= 1 the rows per block (0: automatic).
+ * 256: tiles of 24 and 16 computed rows, for smaller ones, with 256 and up to
+ * 4 rows per block tiles of 14 or 12; 0: the one expected to be fastest),
+ * seg_rows >= 1 the rows per block (0: automatic).
  * Results do not depend on the launch shape. Used by the autotuner. */
 int lb_set_launch(lb_handle* h, int block_x, int seg_rows);
 
@@ -269,8 +270,8 @@ int lb_batch_step(lb_batch* b, int nsteps);
 
 /* Launch shape shared by all instances: block_x 64 (the marching form of
  * lb_set_launch) or 128 (the default: marching or 24-row tiles, whichever is
- * expected to be faster); seg_rows 0 gives every instance a share of one full
- * wave proportional to its cells. */
+ * expected to be faster); seg_rows 0 cuts all instances into segments of about
+ * equal height, the smallest with which their tiles fill the GPU once. */
 int lb_batch_set_launch(lb_batch* b, int block_x, int seg_rows);
 
 /* Persistent mode (the batched boiling curve of Sec. 3.2-3.3 in one launch

@@ -12,8 +12,8 @@ namespace lbgpu {
 
 constexpr int HALO = 5;    // x-halo columns per side recomputed by a block
 constexpr int TILE_COLS = 54;    // columns of a strip (64 less the halos); the marching form's blocks own two
-constexpr int TILE16_ROWS = 6;   // rows a tile of 16 / 24 computed rows writes
-constexpr int TILE24_ROWS = 14;
+constexpr int TILE24_ROWS = 14;  // rows a tile of 24 / 16 / 14 / 12 computed rows writes
+constexpr int TILE16_ROWS = 6, TILE14_ROWS = 4, TILE12_ROWS = 2;
 
 enum { BC_WALLS = 0, BC_TOP_OUTFLOW = 1, BC_PERIODIC = 2 };
 enum : unsigned { ERR_EOS = 1u, ERR_NONFINITE = 2u, ERR_BOUNDS = 4u, ERR_TIMEOUT = 8u };
@@ -24,7 +24,7 @@ struct Acc {
     double q_last;      // q(t) of the last completed step
     double q_sum, q_sum2, q_n;
     double mass;
-    unsigned int count; // bottom blocks that added their partial this step
+    unsigned int count; // unused (part of the saved-state record)
     unsigned int err;   // ERR_* bits
     double pad[2];
 };

@@ -37,17 +37,22 @@ struct TileForm {
         tile_body<NW, K, REC, CG, OUT, QF>(P, C, block, fold, R);
     }
 };
-using Tile16 = TileForm<16, 1>;
 using Tile24 = TileForm<12, 2>;
-static_assert(TileShape<16, 1>::out == TILE16_ROWS && TileShape<12, 2>::out == TILE24_ROWS && TILE_OUT == TILE_COLS &&
+using Tile16 = TileForm<16, 1>;
+using Tile14 = TileForm<14, 1>;
+using Tile12 = TileForm<12, 1>;
+static_assert(TileShape<12, 2>::out == TILE24_ROWS && TileShape<16, 1>::out == TILE16_ROWS &&
+                  TileShape<14, 1>::out == TILE14_ROWS && TileShape<12, 1>::out == TILE12_ROWS && TILE_OUT == TILE_COLS &&
                   MARCH_COLS == 2 * TILE_COLS,
               "the host's launch shapes use these");
 
 // f(form) for the form a launch names (Form in lb_internal.h)
 template <class F>
 auto with_form(int form, F f) {
-    if (form == FORM_TILE16) return f(Tile16{});
     if (form == FORM_TILE24) return f(Tile24{});
+    if (form == FORM_TILE16) return f(Tile16{});
+    if (form == FORM_TILE14) return f(Tile14{});
+    if (form == FORM_TILE12) return f(Tile12{});
     return f(MarchForm{});
 }
 

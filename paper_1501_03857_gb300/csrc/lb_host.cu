@@ -309,7 +309,10 @@ inline int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
 // Column strips and most rows of one pass of a form's block.
 inline bool form_marches(int form) { return form == FORM_MARCH || form == FORM_MARCH6; }
 inline int form_strips(int form, int Lx) { return ceil_div(Lx, form_marches(form) ? 2 * TILE_COLS : TILE_COLS); }
-inline int form_rows(int form) { return form == FORM_TILE16 ? TILE16_ROWS : form == FORM_TILE24 ? TILE24_ROWS : INT32_MAX; }
+inline int form_rows(int form) {
+    constexpr int rows[] = {INT32_MAX, TILE24_ROWS, TILE16_ROWS, TILE14_ROWS, TILE12_ROWS, INT32_MAX};
+    return rows[form];
+}
 
 // About how long a step of `blocks` blocks of seg_rows rows takes, in us, on
 // nsm SMs that hold occ blocks each: the forms' measured times. A tile takes
@@ -319,11 +322,13 @@ inline int form_rows(int form) { return form == FORM_TILE16 ? TILE16_ROWS : form
 // more, being the same work in fewer registers).
 double form_us(int form, long long blocks, int seg_rows, int nsm, int occ) {
     const long long waves = ceil_div(blocks, (long long)nsm * occ);
-    if (form == FORM_TILE16) return 0.5 + 4.1 * waves * ceil_div(seg_rows, TILE16_ROWS);
-    if (form == FORM_TILE24) return 0.8 + 5.7 * waves * ceil_div(seg_rows, TILE24_ROWS);
+    if (!form_marches(form)) {
+        constexpr double wave_us[] = {0.0, 5.85, 4.1, 3.8, 3.4};
+        return 0.5 + wave_us[form] * waves * ceil_div(seg_rows, form_rows(form));
+    }
     const int per_sm = (int)std::min<long long>(occ, ceil_div(blocks, nsm));
     const double iter = form == FORM_MARCH ? 1.75 + 0.13 * per_sm : 1.85 + 0.26 * per_sm;
-    return 1.0 + waves * ceil_div(seg_rows + 2 * HALO, 2) * iter;
+    return 1.0 + waves * ceil_div((long long)seg_rows + 2 * HALO, 2) * iter;
 }
 
 // The launch shape of one form for this grid (seg_rows 0: automatic): a tile
@@ -347,17 +352,19 @@ int form_launch(int form, const lb_grid& g, int seg_rows, int nsm, Launch* out, 
 }
 
 // The launch shape of the fused step for this grid. block_x names the form
-// (64: marching, 128: tiles of 24 rows, 256: tiles of 16 rows); 0 takes the
-// one with the shortest estimate.
+// (64: marching, 128: tiles of 24 rows, 256: tiles of one row per warp, 16 or
+// as few as hold the rows asked for); 0 takes the one with the shortest
+// estimate.
 int compute_launch(const lb_handle* h, int block_x, int seg_rows, Launch* out) {
     int dev = 0, nsm = 0, occ = 0;
     LB_CUDA(cudaGetDevice(&dev), "cudaGetDevice");
     LB_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev), "cudaDeviceGetAttribute");
     if (block_x != 0 && block_x != 64 && block_x != 128 && block_x != 256)
         return fail(LB_E_INVAL, "the fused step takes block_x 64, 128 or 256, not %d", block_x);
-    if (block_x > 0)
-        return form_launch(block_x == 64 ? FORM_MARCH : block_x == 128 ? FORM_TILE24 : FORM_TILE16, h->grid, seg_rows, nsm,
-                           out, &occ);
+    if (block_x > 0) {
+        const int one = seg_rows < 1 || seg_rows > TILE14_ROWS ? FORM_TILE16 : seg_rows > TILE12_ROWS ? FORM_TILE14 : FORM_TILE12;
+        return form_launch(block_x == 64 ? FORM_MARCH : block_x == 128 ? FORM_TILE24 : one, h->grid, seg_rows, nsm, out, &occ);
+    }
     double best = 0;
     for (int form = 0; form < FORM_COUNT; ++form) {
         Launch L;
@@ -416,8 +423,8 @@ int check_device_errors(lb_handle* h) {
     return rc ? rc : report_device_errors(h, h->rec->err);
 }
 
-// Whether p is memory of the current device (else copies go through
-// cudaMemcpy, which takes any address).
+// Whether p is float-aligned memory of the current device (else copies go
+// through cudaMemcpy, which takes any address).
 bool on_this_device(const void* p) {
     cudaPointerAttributes a;
     int dev = -1;
@@ -425,7 +432,7 @@ bool on_this_device(const void* p) {
         cudaGetLastError();
         return false;
     }
-    return a.type == cudaMemoryTypeDevice && a.device == dev;
+    return a.type == cudaMemoryTypeDevice && a.device == dev && (uintptr_t)p % sizeof(float) == 0;
 }
 
 int upload_wall(lb_handle* h) {
@@ -1077,7 +1084,7 @@ BatchTail batch_tail(const lb_batch_desc* d, int n) {
     return T;
 }
 
-// The model constants the step reads from K (step_body, lb_step3.cu): the
+// The model constants the step reads from K (lb_step_batch.cu): the
 // float2 pairs except the wettability and rho_ave, inv_drho, rho_v, cvchi.
 bool same_constants(const StepParams& a, const StepParams& b) {
     for (int k = 0; k < KP_COUNT; ++k)

@@ -10,7 +10,7 @@ namespace lbgpu {
 
 // Forms of the fused step (lb_march.cuh, lb_tile.cuh); the last, marching with
 // six blocks per SM instead of four, for batches only.
-enum Form { FORM_MARCH = 0, FORM_TILE16 = 1, FORM_TILE24 = 2, FORM_COUNT = 3, FORM_MARCH6 = 3 };
+enum Form { FORM_MARCH, FORM_TILE24, FORM_TILE16, FORM_TILE14, FORM_TILE12, FORM_COUNT, FORM_MARCH6 = FORM_COUNT };
 
 // Launch shape of the fused step: nstrips x nseg blocks of seg_rows rows
 // each; block_x threads per block (the form's).

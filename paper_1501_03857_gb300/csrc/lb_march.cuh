@@ -52,7 +52,7 @@ struct MarchSmem {
 };
 
 // The whole step for block `block`: column pair block % npair, segment of
-// P.seg_h rows. C supplies the model constants (see lb_step3.cu); fold: the
+// P.seg_h rows. C supplies the model constants (see lb_step_batch.cu); fold: the
 // previous step's q(t) is still to be folded.
 template <bool REC, bool CG, bool OUT, bool QF>
 __device__ __forceinline__ void march_body(const StepParams& P, const StepParams& C, const int block, const int fold,

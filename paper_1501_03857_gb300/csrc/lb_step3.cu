@@ -3,7 +3,7 @@
 // arithmetic per cell (lb_cell.cuh) and so the same results bit for bit: a
 // marching one for domains that fill the GPU (lb_march.cuh) and a tiled one
 // for smaller ones (lb_tile.cuh, two tile heights); the host picks by the
-// measured times of each (pick_form in lb_host.cu).
+// measured times of each (compute_launch in lb_host.cu).
 #include "lb_forms.cuh"
 
 namespace lbgpu {

@@ -14,11 +14,15 @@
 // lanes 31 and 0.
 //
 // The first rows and columns out are recomputed by every tile that needs
-// them (2.9 cells computed per cell written at 16 rows, 2.0 at 24), which an
-// idle GPU has to spare: on 100 x 100 a step takes 4.6 us with 16 one-row
-// warps (6.6 us with 12 two-row warps), the marching form 15.2 us; on
-// 600 x 150 it is 6.7 us with 24 rows (132 blocks, one wave), 8.4 us with 16
-// (300 blocks), 17.6 us marching. From about 500 x 1000 on marching is
+// them (7.1 cells computed per cell written at 12 rows, 4.1 at 14, 3.2 at 16,
+// 2.0 at 24), which an idle GPU has to spare. A tile's time is its warps' work
+// on one SM plus the chain of stages, so on a domain that leaves SMs empty
+// smaller tiles are faster while they still come to one wave: a step of
+// 100 x 100 takes 4.25 us with 12 one-row warps (100 blocks), 4.6 with 14
+// (50), 4.9 with 16 (34), 6.5 with 12 two-row warps (16), and 15.2 us
+// marching; 300 x 100 takes 7.3 us with 12 (300 blocks, two waves), 4.8 with
+// 14 (150) and 5.0 with 16; 600 x 150 6.7 us with 24 rows (132 blocks), 8.4
+// us with 16 (300), 17.6 us marching. From about 500 x 1000 on marching is
 // faster (24.8 against 28.3 us).
 #pragma once
 
@@ -333,7 +337,7 @@ __device__ __forceinline__ void tile_rows(const StepParams& P, const StepParams&
 
 // The whole step for block `block`: strip block % nstrips, and the rows of its
 // segment (P.seg_h, normally one tile's). K = C supplies the model constants
-// (see lb_step3.cu); fold: the previous step's q(t) is still to be folded.
+// (see lb_step_batch.cu); fold: the previous step's q(t) is still to be folded.
 template <int NW, int K, bool REC, bool CG, bool OUT, bool QF>
 __device__ __forceinline__ void tile_body(const StepParams& P, const StepParams& C, const int block, const int fold,
                                           const RecomputeOut* R) {

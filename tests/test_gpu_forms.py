@@ -1,5 +1,5 @@
-"""The forms of the fused step (marching, tiles of 24 and of 16 rows; block_x
-64, 128, 256) at the sizes where they can go wrong: one column or row short
+"""The forms of the fused step (marching, tiles of 24 rows and of 16, 14 and 12;
+block_x 64, 128, 256) at the sizes where they can go wrong: one column or row short
 of, at and past a strip, a pair of strips and a tile, domains narrower than a
 strip, and segments that a block walks tile by tile. Every form gives the same
 bits, heat flux included, and one step agrees with the FP64 oracle within the
@@ -14,7 +14,7 @@ from parity_util import norm_err, oracle_params, run_oracle, theta_err
 
 pytestmark = pytest.mark.gpu
 
-FORMS = ((64, 0), (128, 0), (256, 0), (64, 1), (64, 9), (128, 5), (128, 40), (256, 17))
+FORMS = ((64, 0), (128, 0), (256, 0), (256, 2), (256, 3), (64, 1), (64, 9), (128, 5), (128, 40), (256, 17))
 # (Lx, Ly, bc, ghost, isothermal)
 CASES = [(53, 5, 0, False, False), (54, 6, 1, False, False), (55, 7, 0, True, False), (107, 13, 0, False, False),
          (108, 14, 2, False, False), (109, 15, 1, True, False), (3, 27, 0, False, False), (64, 28, 2, False, True),
