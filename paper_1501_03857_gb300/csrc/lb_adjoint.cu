@@ -5,9 +5,10 @@
 //
 // Forward intermediates of step n are recomputed from the stored state
 // (f*^n, theta^n) by the fused step itself in its recompute mode
-// (lb_step3.cu, RecomputeOut), which the adjoint driver runs while it
+// (lb_step_rec.cu, RecomputeOut), which the adjoint driver runs while it
 // replays a checkpoint segment. The reverse passes then transpose each part
-// of the step in the opposite order:
+// of the step in the opposite order, on large domains in two launches, on
+// small ones in one (rev_tile, lb_rev_tile.cuh):
 //
 //   RK4 of Eq. 18 (stage 4 .. 1)   -> lambda_theta, lambda of the per-cell
 //   and the coefficients              coefficients (ax, ay, cA, cB), then
@@ -166,250 +167,252 @@ __device__ __forceinline__ void rev_coef_vals(const StepParams& P, const AdjFiel
 // Each RK stage of Eq. 18 (stage 4 .. 1) transposed and then the
 // coefficients (rev_coef_vals), cell by cell, in one pass over the domain: a
 // block of RT_BD threads owns RT_BD - 2 RT_HALO output columns and a segment
-// of rows and marches up the segment one row per iteration, each thread one
+// of rows and marches up the segment two rows per iteration, each thread one
 // column:
 //
-//   S  row L    : mu4 = lambda_theta'/6 (fluid rows), ax, ay into shared
-//                 rings; u4, u3 (row L), u2 (row L - 2), theta (row L - 3);
-//                 cA, cB, lambda-bar (own column)
-//   R4 row L-1  : stage 4 transposed (rows L-2..L) -> mu3
-//   R3 row L-2  : stage 3 transposed -> mu2
-//   R2 row L-3  : stage 2 transposed -> mu1
-//   R1 row L-4  : stage 1 transposed; the cell's coefficient adjoints are
-//                 complete: lambda of grad rho, div v, rho, v, theta out
+//   S  rows L, L+1   : mu4 = lambda_theta'/6 (fluid rows), ax, ay, u4 into
+//                      shared rows; u3, u2, theta one, two, three rows
+//                      behind; cA, cB (rows L-1, L), lambda-bar (own column)
+//   R4 rows L-1, L   : stage 4 transposed -> mu3
+//   R3 rows L-2, L-1 : stage 3 transposed -> mu2
+//   R2 rows L-3, L-2 : stage 2 transposed -> mu1
+//   R1 rows L-4, L-3 : stage 1 transposed; the cells' coefficient adjoints are
+//                      complete: lambda of grad rho, div v, rho, v, theta out
 //
 // A stage's lambda_u at x gathers c_d(x - d) mu(x - d) over the 9 cells
 // around x, with c_d(s) = ax(s) wx(d) + ay(s) wy(d) + chi wl(d) the
 // isotropic stencils of Sec. 2. With the first-derivative weights odd in d
 // that is lambda_u = -Dx[ax mu] - Dy[ay mu] + chi Lap[mu]: the forward
 // stencils applied to the products, formed at each neighbour from the ax,
-// ay and mu rings (ax, ay are the same for all four stages, so two rings
-// serve them all). Each stage reaches one column further out: 4
-// halo columns per side. The per-cell accumulators (coefficient adjoints,
-// lambda_theta) ride along with their row in registers. Walls in y only
-// (the adjoint's supported case). (Measured: this scalar form with 4 warps
-// per block runs 1.5 x faster than a paired-FP32 form over two strips,
-// whose shared rings allowed only 10 warps per SM; rings of the products
-// ax mu, ay mu per stage took 43.5 KB per block, 5 blocks per SM. Steady
-// iterations without range and wall tests: 95 registers, 5 blocks per SM,
-// and the 2048^2 reverse step 0.374 ms instead of 0.414; held to 7 blocks
-// per SM, 72 registers with a small spill, 0.414. Packing each stage's u,
-// mu, ax mu and ay mu into one float4 ring, products formed by the thread
-// that forms mu, so that a neighbour is one 16-byte load (9 loads and 2
-// products per stage instead of 33 and 12): 0.404 ms at 4 blocks per SM
-// (128 registers), 0.446 at 5 (96 registers with a spill), against 0.363
-// for this form: a 16-byte load of a warp takes 4 shared-memory wavefronts
-// and the partial float4 stores at a 16-byte stride as many, more than the
-// 33 conflict-free 4-byte loads they replace.)
-// ring rows: RT_R for mu and u (3 rows read, one written per iteration),
-// RT_RA for ax, ay (read by all four stages: rows L-5..L)
-constexpr int RT_BD = 128, RT_HALO = 4, RT_W = RT_BD + 2, RT_R = 4, RT_RA = 8;
-constexpr int RT_SMN = (8 * RT_R + 2 * RT_RA) * RT_W + 3 * RT_R * RT_BD;  // floats of shared memory
+// ay and mu rows (ax, ay are the same for all four stages). Every stencil is a
+// sum of one term per row, and a row's terms serve the three rows around it:
+// a stage reads only the two rows its predecessor has just finished and keeps
+// the terms of the two before in registers (22 shared loads per stage and two
+// rows, where nine-point sums row by row took 62). Each stage reaches one
+// column further out: 4 halo columns per side. The per-cell accumulators
+// (coefficient adjoints, lambda_theta) ride along with their row in
+// registers: a stage's first row goes on to the next stage at once, the
+// second in the next iteration. Walls in y only (the adjoint's supported
+// case).
+//
+// What bounds it: the shared-memory path and fixed-latency waits at twelve
+// warps per SM (165 registers). 2048^2: 83 us per launch, 105 us for one row
+// per iteration with nine-point sums (20 warps); 69 bytes per cell, 43 us from
+// HBM. Held to 128 registers (16 warps, 120 bytes of spill) it takes as long as
+// that; blocks of 64 and 192 threads are 1-2 us slower, of 256 17 us; loading
+// the next rows after the first, second or third stage instead of before the
+// first 3, 6 and 11 us slower.
+constexpr int RT_BD = 128, RT_MINB = 3, RT_HALO = 4, RT_W = RT_BD + 2, RT_RA = 8;
+// shared floats: mu of each stage and u4, u3, u2 (two rows: written and read
+// in one iteration), theta (four: its reader and the next iteration's writer
+// have no barrier between them), ax, ay (eight: rows L-3 .. L+1 are read),
+// cA, cB, lambda-bar of the own column (rows L-4 .. L+1)
+constexpr int RT_TH = 14 * RT_W, RT_AX = RT_TH + 4 * RT_W, RT_AY = RT_AX + RT_RA * RT_W, RT_OWN = RT_AY + RT_RA * RT_W;
+constexpr int RT_SMN = RT_OWN + 3 * RT_RA * RT_BD;
 
-__global__ void __launch_bounds__(RT_BD) rev_thermal_fused(const StepParams P, AdjFields A, int seg_h) {
+__global__ void __launch_bounds__(RT_BD, RT_MINB) rev_thermal_fused(const StepParams P, AdjFields A, int seg_h) {
     extern __shared__ float rt_sm[];
-    float* const sMU = rt_sm;                   // per stage (4, 3, 2, 1 -> 0..3): [4][RT_R][RT_W]
-    float* const sU = sMU + 4 * RT_R * RT_W;    // u4, u3, u2, theta: [4][RT_R][RT_W]
-    float* const sAX = sU + 4 * RT_R * RT_W;    // ax, ay: [2][RT_RA][RT_W]
-    float* const sOWN = sAX + 2 * RT_RA * RT_W;  // cA, cB, lambda-bar: [3][RT_R][RT_BD]
-    constexpr int SMN = RT_SMN;
-    for (int i = threadIdx.x; i < SMN; i += RT_BD) rt_sm[i] = 0.f;
+    for (int i = threadIdx.x; i < RT_SMN; i += RT_BD) rt_sm[i] = 0.f;
 
     const int Lx = P.Lx, Ly = P.Ly, pitch = P.pitch;
     const int nout = RT_BD - 2 * RT_HALO;
     const int nstrips = (Lx + nout - 1) / nout;
     const int strip = blockIdx.x % nstrips, seg = blockIdx.x / nstrips;
-    const int lc = threadIdx.x, s = lc + 1;
+    const int lc = threadIdx.x;
     int x = (strip * nout - RT_HALO + lc) % Lx;
     if (x < 0) x += Lx;
     const bool out = lc >= RT_HALO && lc < RT_HALO + nout && strip * nout + lc - RT_HALO < Lx;
     const int ys = seg * seg_h, ye = min(ys + seg_h, Ly);
     const int lo = max(ys - RT_HALO, 0), hi = min(ye + RT_HALO - 1, Ly - 1);  // rows loaded
-    const float chi = P.chi;
-    // this thread's slot of row L - j in the rings, j = 0..5, set at the
-    // start of iteration L; a ring field is a fixed offset from it, so every
-    // shared access is a register plus an immediate
-    float* p4[6] = {};  // mu and u rings (RT_R slots)
-    float* p8[6] = {};  // ax, ay rings (RT_RA slots)
-    float* q4[6] = {};  // own-column values (RT_R slots)
-    auto own = [&](int f, int j) -> float& { return q4[j][f * RT_R * RT_BD]; };  // 0 cA, 1 cB, 2 lambda-bar
-    auto mu = [&](int k, int j) { return p4[j] + k * RT_R * RT_W; };
-    auto uu = [&](int k, int j) { return p4[j] + (4 + k) * RT_R * RT_W; };
-    auto aring = [&](int k, int j) { return p8[j] + k * RT_RA * RT_W; };  // 0 ax, 1 ay
-    float acc_ax[4], acc_ay[4], acc_cA[4], acc_cB[4], acc_th[4];  // index k: the row stage k worked on
+    const float chi6 = P.chi * (1.f / 6.f);
+    float* const sm = rt_sm + lc + 1;
+    // (L - lo is even: row L - j of a two-row ring is its slot j & 1)
+    auto mu = [&](int k, int j) { return sm + (2 * k + (j & 1)) * RT_W; };
+    float* pa[5];  // ax of rows L + 1 - j, j = 0 .. 4 (ay: RT_AY - RT_AX further on)
+    float* pt[2];  // theta of rows L - 2, L - 3
+    float* po[6];  // own-column values of rows L + 1 - j: cA, then cB and lambda-bar
+    auto uu = [&](int k, int j) { return k < 3 ? sm + (8 + 2 * k + (j & 1)) * RT_W : pt[j - 2]; };
+    constexpr int CB = RT_RA * RT_BD, LB = 2 * RT_RA * RT_BD;
+
+    // Per stage, of the two rows before those it is about to read: the terms of
+    // 12 Dx[ax mu], 12 Dy[ay mu], 12 Dx[u], 12 Dy[u] of both (m, c), of 6
+    // Lap[mu] of the first, and mu's sides and the own mu and u of the second
+    struct Rows {
+        float dm, dc, sm, sc, em, side, mu0, xm, xc, tm, tc, u0;
+    } rows[4];
+    struct Sum {
+        float ax, ay, cA, cB, th;
+    } carry[4];  // [k]: of the first row stage k works on next
 #pragma unroll
-    for (int k = 0; k < 4; ++k) acc_ax[k] = acc_ay[k] = acc_cA[k] = acc_cB[k] = acc_th[k] = 0.f;
+    for (int k = 0; k < 4; ++k) {
+        rows[k] = Rows{};
+        carry[k] = Sum{};
+    }
     __syncthreads();
 
-    // stage k (0: stage 4 .. 3: stage 1) at row r = L - 1 - k (slot k + 1;
-    // its rows r - 1 and r + 1 are slots k + 2 and k); in a steady iteration
-    // (S) no row of any stage is a wall row or next to one
-    auto stage = [&](const int k, const int r, auto steady) {
+    // Stage k (0: stage 4 .. 3: stage 1) on rows r = L - 1 - k and r + 1; in a
+    // steady iteration (S) no row of any stage is a wall row or next to one.
+    // a, b: the two rows' sums so far, and with this stage.
+    auto stage = [&](const int k, const int r, Sum& a, Sum& b, auto steady) {
         constexpr bool S = decltype(steady)::value;
-        const bool wall = !S && (r == 0 || r == Ly - 1);
-        // rows beyond the walls hold no cell: their products are 0
-        const bool hm = S || r - 1 >= 0, hp = S || r + 1 < Ly;
-        const int jm = k + 2, jc = k + 1, jp = k;
-        const float* xm = aring(0, jm);
-        const float* xc = aring(0, jc);
-        const float* xp = aring(0, jp);
-        const float* ym = aring(1, jm);
-        const float* yp = aring(1, jp);
-        const float* mm = mu(k, jm);
-        const float* mc = mu(k, jc);
-        const float* mp = mu(k, jp);
-        // 12 Dx[ax mu], 12 Dy[ay mu], 6 Lap[mu] (unweighted sums of the stencils)
-        float dxp = 4.f * (xc[1] * mc[1] - xc[-1] * mc[-1]), dyp = 0.f;
-        float lap = -20.f * mc[0] + 4.f * (mc[1] + mc[-1]);
-        if (hm) {
-            dxp += xm[1] * mm[1] - xm[-1] * mm[-1];
-            dyp -= 4.f * ym[0] * mm[0] + ym[1] * mm[1] + ym[-1] * mm[-1];
-            lap += 4.f * mm[0] + mm[1] + mm[-1];
+        Rows& R = rows[k];
+        // the two new rows' terms (rows beyond the walls hold no cell: theirs are 0)
+        float d[2], s[2], side[2], m0[2], ux[2], ut[2], u0[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int j = k - i;  // row L - j = r + 1 + i
+            const float* m = mu(k, j);
+            const float* ax = pa[j + 1];
+            const float* ay = ax + (RT_AY - RT_AX);
+            const float* u = uu(k, j);
+            const float ml = m[-1], mr = m[1];
+            m0[i] = m[0];
+            side[i] = ml + mr;
+            d[i] = ax[1] * mr - ax[-1] * ml;
+            s[i] = 4.f * ay[0] * m0[i] + ay[1] * mr + ay[-1] * ml;
+            u0[i] = u[0];
+            ux[i] = u[1] - u[-1];
+            ut[i] = 4.f * u0[i] + u[1] + u[-1];
+            if (!S && (r + 1 + i < 0 || r + 1 + i >= Ly)) m0[i] = side[i] = d[i] = s[i] = 0.f;
         }
-        if (hp) {
-            dxp += xp[1] * mp[1] - xp[-1] * mp[-1];
-            dyp += 4.f * yp[0] * mp[0] + yp[1] * mp[1] + yp[-1] * mp[-1];
-            lap += 4.f * mp[0] + mp[1] + mp[-1];
+        const float ec = 4.f * R.mu0 + R.side, e0 = 4.f * m0[0] + side[0], e1 = 4.f * m0[1] + side[1];
+        // row r: rows m, c and the first new one; row r + 1: c and both new ones
+        float lu[2] = {-(4.f * R.dc + R.dm + d[0] + s[0] - R.sm) * (1.f / 12.f) + chi6 * (4.f * R.side - 20.f * R.mu0 + R.em + e0),
+                       -(4.f * d[0] + R.dc + d[1] + s[1] - R.sc) * (1.f / 12.f) + chi6 * (4.f * side[0] - 20.f * m0[0] + ec + e1)};
+        const float mm[2] = {R.mu0, m0[0]}, th[2] = {R.u0, u0[0]};
+        const float gx[2] = {4.f * R.xc + R.xm + ux[0], 4.f * ux[0] + R.xc + ux[1]}, gy[2] = {ut[0] - R.tm, ut[1] - R.tc};
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const bool wall = !S && (r + i == 0 || r + i == Ly - 1);
+            const float* o = po[k + 2 - i];  // row r + i = L + 1 - (k + 2 - i)
+            const float lbar = o[LB];
+            Sum& q = i ? b : a;
+            if (k == 0) q = Sum{0.f, 0.f, 0.f, 0.f, lbar};
+            if (S || !wall) {
+                const float m = mm[i], T = P.Ts + th[i];
+                const float rsq = rsqrt_a(T);
+                const float dphi = P.k1k1 - P.k0k1 * rsq;
+                const float d2phi = 0.5f * P.k0k1 * (rsq * rsq * rsq);
+                const float cA = o[0], cB = o[CB];
+                lu[i] += (-(cA - cB * dphi) + T * cB * d2phi) * m;
+                const float m12 = m * (1.f / 12.f);
+                q.ax += gx[i] * m12;
+                q.ay += gy[i] * m12;
+                q.cA -= T * m;
+                q.cB += T * dphi * m;
+            }
+            q.th += lu[i];
+            if (k < 3) {  // the next stage's mu = a lambda-bar + b lambda_u on fluid rows
+                const float ab = k == 2 ? 1.f / 6.f : 1.f / 3.f, bb = k == 0 ? 1.f : 0.5f;
+                *mu(k + 1, k + 1 - i) = wall ? 0.f : ab * lbar + bb * lu[i];
+            }
         }
-        float lu = -(dxp + dyp) * (1.f / 12.f) + chi * (1.f / 6.f) * lap;
-        const float m = mc[0];
-        float lax = 0.f, lay = 0.f, lcA = 0.f, lcB = 0.f;
-        if (!wall && m != 0.f) {
-            const float* um = uu(k, jm);
-            const float* uc = uu(k, jc);
-            const float* up = uu(k, jp);
-            const float T = P.Ts + uc[0];
-            const float rsq = rsqrt_a(T);
-            const float dphi = P.k1k1 - P.k0k1 * rsq;
-            const float d2phi = 0.5f * P.k0k1 * (rsq * rsq * rsq);
-            const float cA = own(0, jc), cB = own(1, jc);
-            lu += (-(cA - cB * dphi) + T * cB * d2phi) * m;
-            const float ux = (uc[1] - uc[-1]) * (1.f / 3.f) + ((up[1] - um[-1]) + (um[1] - up[-1])) * (1.f / 12.f);
-            const float uy = (up[0] - um[0]) * (1.f / 3.f) + ((up[1] - um[-1]) + (up[-1] - um[1])) * (1.f / 12.f);
-            lax = ux * m;
-            lay = uy * m;
-            lcA = -T * m;
-            lcB = T * dphi * m;
-        }
-        if (k == 0) {
-            acc_ax[0] = lax;
-            acc_ay[0] = lay;
-            acc_cA[0] = lcA;
-            acc_cB[0] = lcB;
-            acc_th[0] = own(2, jc) + lu;
-        } else {
-            acc_ax[k] += lax;
-            acc_ay[k] += lay;
-            acc_cA[k] += lcA;
-            acc_cB[k] += lcB;
-            acc_th[k] += lu;
-        }
-        if (k < 3) {  // the next stage's mu = a lambda-bar + b lambda_u on fluid rows
-            const float ab = k == 2 ? 1.f / 6.f : 1.f / 3.f, bb = k == 0 ? 1.f : 0.5f;
-            *mu(k + 1, jc) = wall ? 0.f : ab * own(2, jc) + bb * lu;
-        }
+        R = Rows{d[0], d[1], s[0], s[1], e0, side[1], m0[1], ux[0], ux[1], ut[0], ut[1], u0[1]};
     };
 
-    // the inputs of iteration L, loaded one iteration ahead (their latency is
-    // hidden behind the stages): lambda_theta', ax, ay, u4, u3 of row L, rho
-    // and div v of row L - 1 (for cA, cB), u2 of row L - 2, theta of row
-    // L - 3, and rho, div v, grad rho of row L - 4 (the output row)
-    float n_lin = 0.f, n_ax = 0.f, n_ay = 0.f, n_u4 = 0.f, n_u3 = 0.f, n_r1 = 0.f, n_d1 = 0.f, n_u2 = 0.f, n_th = 0.f;
-    float n_rho = 0.f, n_dv = 0.f, n_drx = 0.f, n_dry = 0.f;
+    // the inputs of an iteration, loaded one iteration ahead (their latency is
+    // hidden behind the stages): lambda_theta', ax, ay, u4 of rows L, L + 1, rho
+    // and div v (for cA, cB) and u3 of rows L - 1, L, u2 and theta one and two
+    // rows behind
+    float n_lin[2] = {}, n_ax[2] = {}, n_ay[2] = {}, n_u4[2] = {}, n_u3[2] = {}, n_r[2] = {}, n_d[2] = {}, n_u2[2] = {}, n_th[2] = {};
     auto prefetch = [&](int L, auto steady) {
         constexpr bool S = decltype(steady)::value;
-        if (S || L <= hi) {
-            const int i = L * pitch + x;
-            n_lin = LB_LD(A.lt_in, i, P.plane);
-            n_ax = LB_LD(A.ax, i, P.plane);
-            n_ay = LB_LD(A.ay, i, P.plane);
-            n_u4 = LB_LD(A.u4, i, P.plane);
-            n_u3 = LB_LD(A.u3, i, P.plane);
-        }
-        if (S || (L - 1 >= lo && L - 1 <= hi)) {
-            const int i = (L - 1) * pitch + x;
-            n_r1 = LB_LD(A.rho, i, P.plane);
-            n_d1 = LB_LD(A.divv, i, P.plane);
-        }
-        if (S || (L - 2 >= lo && L - 2 <= hi)) n_u2 = LB_LD(A.u2, (L - 2) * pitch + x, P.plane);
-        if (S || (L - 3 >= lo && L - 3 <= hi)) n_th = LB_LD(A.theta, (L - 3) * pitch + x, P.plane);
-        if ((S || (L - 4 >= ys && L - 4 < ye)) && out) {
-            const int i = (L - 4) * pitch + x;
-            n_rho = LB_LD(A.rho, i, P.plane);
-            n_dv = LB_LD(A.divv, i, P.plane);
-            n_drx = LB_LD(A.drx, i, P.plane);
-            n_dry = LB_LD(A.dry, i, P.plane);
+        auto in = [&](int r) { return S || (r >= lo && r <= hi); };
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int o = (L + i) * pitch + x;
+            if (in(L + i)) {
+                n_lin[i] = LB_LD(A.lt_in, o, P.plane);
+                n_ax[i] = LB_LD(A.ax, o, P.plane);
+                n_ay[i] = LB_LD(A.ay, o, P.plane);
+                n_u4[i] = LB_LD(A.u4, o, P.plane);
+            }
+            if (in(L + i - 1)) {
+                n_u3[i] = LB_LD(A.u3, o - pitch, P.plane);
+                n_r[i] = LB_LD(A.rho, o - pitch, P.plane);
+                n_d[i] = LB_LD(A.divv, o - pitch, P.plane);
+            }
+            if (in(L + i - 2)) n_u2[i] = LB_LD(A.u2, o - 2 * pitch, P.plane);
+            if (in(L + i - 3)) n_th[i] = LB_LD(A.theta, o - 3 * pitch, P.plane);
         }
     };
     prefetch(lo, std::false_type{});
-    // one row iteration L; in a steady one (S) every row it touches (L - 5 ..
-    // L + 1) is loaded, off the walls and not next to them, and the output
-    // row is the block's own, so the range and wall tests are compiled out
+    // one iteration, rows L and L + 1; in a steady one (S) every row it touches
+    // (L - 4 .. L + 3) is loaded and off the walls, and the output rows are the
+    // block's own, so the range and wall tests are compiled out
     auto iter = [&](const int L, auto steady) {
         constexpr bool S = decltype(steady)::value;
+        const int l = L - lo + 1 + RT_RA;
 #pragma unroll
         for (int j = 0; j < 6; ++j) {
-            p4[j] = rt_sm + ((L - j) & (RT_R - 1)) * RT_W + s;
-            p8[j] = sAX + ((L - j) & (RT_RA - 1)) * RT_W + s;
-            q4[j] = sOWN + ((L - j) & (RT_R - 1)) * RT_BD + lc;
-        }
-        // ---- S: the prefetched row into the rings, then the next one's loads
-        if (S || L <= hi) {
-            const bool wall = !S && (L == 0 || L == Ly - 1);
-            *mu(0, 0) = wall ? 0.f : n_lin * (1.f / 6.f);
-            *aring(0, 0) = n_ax;
-            *aring(1, 0) = n_ay;
-            own(2, 0) = wall ? 0.f : n_lin;
-            *uu(0, 0) = n_u4;
-            *uu(1, 0) = n_u3;
-        }
-        if (S || (L - 1 >= lo && L - 1 <= hi)) {  // cA, cB of row L - 1 (stage 4 there next)
-            // the coefficients of the source term as the step forms them (Eq. 18):
-            // cA = div v R / (c_v (1 - b rho)), cB = div v a rho / (c_v (1 + 2 b rho - b^2 rho^2))
-            const float br = P.b * n_r1;
-            own(0, 1) = n_d1 * P.R * P.inv_cv * rcp_a(1.f - br);
-            own(1, 1) = n_d1 * P.a * n_r1 * P.inv_cv * rcp_a(fmaf(br, 2.f - br, 1.f));
-        }
-        if (S || (L - 2 >= lo && L - 2 <= hi)) *uu(2, 2) = n_u2;
-        if (S || (L - 3 >= lo && L - 3 <= hi)) *uu(3, 3) = n_th;
-        const float o_rho = n_rho, o_dv = n_dv, o_drx = n_drx, o_dry = n_dry;  // row L - 4
-        prefetch(L + 1, steady);
-        __syncthreads();
-        if (S || (L - 1 >= lo && L - 1 <= hi)) stage(0, L - 1, steady);
-        __syncthreads();
-        if (S || (L - 2 >= lo && L - 2 <= hi)) stage(1, L - 2, steady);
-        __syncthreads();
-        if (S || (L - 3 >= lo && L - 3 <= hi)) stage(2, L - 3, steady);
-        __syncthreads();
-        const int r = L - 4;
-        if (S || (r >= ys && r < ye)) {
-            stage(3, r, steady);
-            if (out) {
-                const int i = r * pitch + x;
-                LB_ST(A.lth, i, P.plane, acc_th[3]);
-                rev_coef_vals(P, A, i, !S && (r == 0 || r == Ly - 1), acc_ax[3], acc_ay[3], acc_cA[3], acc_cB[3],
-                              o_rho, o_dv, o_drx, o_dry);
-                if (!S && r == 0) LB_ADD(A.dTb, x, P.pitch, (double)LB_LD(A.lt_in, i, P.plane));
-            }
+            if (j < 5) pa[j] = sm + RT_AX + ((l - j) & (RT_RA - 1)) * RT_W;
+            po[j] = rt_sm + RT_OWN + ((l - j) & (RT_RA - 1)) * RT_BD + lc;
         }
 #pragma unroll
-        for (int k = 3; k > 0; --k) {
-            acc_ax[k] = acc_ax[k - 1];
-            acc_ay[k] = acc_ay[k - 1];
-            acc_cA[k] = acc_cA[k - 1];
-            acc_cB[k] = acc_cB[k - 1];
-            acc_th[k] = acc_th[k - 1];
+        for (int j = 0; j < 2; ++j) pt[j] = sm + RT_TH + ((l - 3 - j) & 3) * RT_W;
+        // ---- S: the prefetched rows into the rings, then the next ones' loads
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const bool wall = !S && (L + i == 0 || L + i == Ly - 1);
+            *mu(0, -i) = wall ? 0.f : n_lin[i] * (1.f / 6.f);
+            *pa[1 - i] = n_ax[i];
+            pa[1 - i][RT_AY - RT_AX] = n_ay[i];
+            po[1 - i][LB] = wall ? 0.f : n_lin[i];
+            *uu(0, -i) = n_u4[i];
+            *uu(1, 1 - i) = n_u3[i];
+            *uu(2, 2 - i) = n_u2[i];
+            *uu(3, 3 - i) = n_th[i];
+            // the coefficients of the source term of rows L - 1, L as the step forms them (Eq. 18):
+            // cA = div v R / (c_v (1 - b rho)), cB = div v a rho / (c_v (1 + 2 b rho - b^2 rho^2))
+            const float br = P.b * n_r[i];
+            po[2 - i][0] = n_d[i] * P.R * P.inv_cv * rcp_a(1.f - br);
+            po[2 - i][CB] = n_d[i] * P.a * n_r[i] * P.inv_cv * rcp_a(fmaf(br, 2.f - br, 1.f));
         }
+        // the output rows' rho, div v, grad rho
+        float o_rho[2] = {}, o_dv[2] = {}, o_drx[2] = {}, o_dry[2] = {};
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int r = L - 4 + i;
+            if (out && (S || (r >= ys && r < ye))) {
+                const int o = r * pitch + x;
+                o_rho[i] = LB_LD(A.rho, o, P.plane);
+                o_dv[i] = LB_LD(A.divv, o, P.plane);
+                o_drx[i] = LB_LD(A.drx, o, P.plane);
+                o_dry[i] = LB_LD(A.dry, o, P.plane);
+            }
+        }
+        prefetch(L + 2, steady);
         __syncthreads();
+        Sum a, b;
+        stage(0, L - 1, a, b, steady);
+#pragma unroll
+        for (int k = 1; k < 4; ++k) {
+            __syncthreads();
+            const Sum c = carry[k];
+            carry[k] = b;
+            b = a;
+            a = c;
+            stage(k, L - 1 - k, a, b, steady);
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int r = L - 4 + i;
+            if (out && (S || (r >= ys && r < ye))) {
+                const Sum& q = i ? b : a;
+                const int o = r * pitch + x;
+                LB_ST(A.lth, o, P.plane, q.th);
+                rev_coef_vals(P, A, o, !S && (r == 0 || r == Ly - 1), q.ax, q.ay, q.cA, q.cB, o_rho[i], o_dv[i], o_drx[i],
+                              o_dry[i]);
+                if (!S && r == 0) LB_ADD(A.dTb, x, P.pitch, (double)LB_LD(A.lt_in, o, P.plane));
+            }
+        }
     };
-    // steady iterations: the rows L - 5 .. L + 1 lie in [1, Ly - 2] and in
-    // the loaded rows, the output rows of L and L + 1 in [ys, ye)
-    const int Ls = max(max(ys + 4, 6), lo + 1);
-    const int Le = min(min(hi - 1, Ly - 2), ye + 2) + 1;
+    // steady iterations: L - 4 >= 1 and ys, L + 3 <= hi and Ly - 2, L - 3 < ye
+    const int Ls = max(ys + 4, 5), Le = min(min(hi - 3, Ly - 5), ye + 2);
     int L = lo;
-    for (; L < Ls; ++L) iter(L, std::false_type{});
-    for (; L < Le; ++L) iter(L, std::true_type{});
-    for (; L <= hi + RT_HALO; ++L) iter(L, std::false_type{});
+    for (; L < Ls; L += 2) iter(L, std::false_type{});
+    for (; L <= Le; L += 2) iter(L, std::true_type{});
+    for (; L - 4 < ye; L += 2) iter(L, std::false_type{});
 }
 
 constexpr int RV_NW = 12, RV_K = 2, RV_SMEM = RevShape2<RV_NW, RV_K>::slots * (int)sizeof(float2);
@@ -903,8 +906,7 @@ cudaError_t adjoint_grads_finish(const StepParams& P, void* work, const float* l
 
 // One reverse step: state (fstar, theta) of level n and the intermediates R
 // of the step from it, lambda of level n+1 in (lf_in with lr_in, lt_in),
-// lambda of level n out (lf_out with lr_out, lt_out); lq = dJ/dq(t_n). L is a dual-strip
-// launch shape matching P (nout, nstrips, seg_h) for the recompute.
+// lambda of level n out (lf_out with lr_out, lt_out); lq = dJ/dq(t_n).
 cudaError_t adjoint_reverse_step(const StepParams& P, const RecomputeOut& R, void* work, const float* fstar,
                                  const float* theta, const float* lf_in, const float* lt_in, const float* lr_in,
                                  float* lf_out, float* lt_out, float* lr_out, float lq, cudaStream_t st) {
@@ -956,11 +958,11 @@ cudaError_t adjoint_reverse_step(const StepParams& P, const RecomputeOut& R, voi
     if (RS.e != cudaSuccess) return RS.e;
     const int nsm = RS.nsm, occ_t = RS.occ_t, occ_f = RS.occ_f;
     const int tiles = (P.Lx + RV_COLS - 1) / RV_COLS * rev_tiles<RevShape2<RV_NW, RV_K>>(P.Ly);
-    // the tiles while they come to three waves at most (one block per SM, 13
-    // us a wave): the marching kernels take 26 us at the least and overtake
-    // at four waves (512^2: 62 us against 66 with the forward step; 517 x
-    // 1003, six waves: 114 against 93)
-    if (tiles <= 3 * nsm) {
+    // the tiles while they come to two waves at most (one block per SM, 13 us a
+    // wave; with the forward step, us per step: 400^2, two waves, 45.3 either
+    // way; 512 x 400, three, 55.9 against 49.5 marching; 512^2 63.7 against
+    // 57.8; 600 x 450 64.0 against 56.8)
+    if (tiles <= 2 * nsm) {
         StepParams Q = P;  // the pull reads the state through the parameters
         Q.f_in = fstar;
         Q.th_in = theta;
