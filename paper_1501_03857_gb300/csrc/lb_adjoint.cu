@@ -958,11 +958,11 @@ cudaError_t adjoint_reverse_step(const StepParams& P, const RecomputeOut& R, voi
     if (RS.e != cudaSuccess) return RS.e;
     const int nsm = RS.nsm, occ_t = RS.occ_t, occ_f = RS.occ_f;
     const int tiles = (P.Lx + RV_COLS - 1) / RV_COLS * rev_tiles<RevShape2<RV_NW, RV_K>>(P.Ly);
-    // the tiles while they come to two waves at most (one block per SM, 13 us a
-    // wave; with the forward step, us per step: 400^2, two waves, 45.3 either
-    // way; 512 x 400, three, 55.9 against 49.5 marching; 512^2 63.7 against
-    // 57.8; 600 x 450 64.0 against 56.8)
-    if (tiles <= 2 * nsm) {
+    // the tiles while they come to one wave (one block per SM, 13 us; a step of
+    // the whole adjoint, us, tiles against marching: 600 x 150 28.8 and 34.6,
+    // 320 x 256 28.2 and 34.5, one wave; 400 x 300 46.0 and 41.6, 400^2 45.3 and
+    // 45.2, two waves; 512 x 400 55.9 and 49.6, three)
+    if (tiles <= nsm) {
         StepParams Q = P;  // the pull reads the state through the parameters
         Q.f_in = fstar;
         Q.th_in = theta;
