@@ -104,8 +104,10 @@ __global__ void macro_pass2(const StepParams P, const float* __restrict__ scr, f
 // threads marches up a segment of rows, one column per thread, the outer two
 // halo. psi of the last rows sits in a four-row shared ring (one barrier per
 // row); rho and the momentum sums of a row wait in registers for the row
-// above it. Bound by HBM: ten planes in, four out, against 48 more bytes per
-// cell when rho, psi and j went through scratch planes between two kernels.
+// above it. Ten planes in, four out, 48 bytes per cell less than with rho, psi
+// and j in scratch planes between two kernels: 57 us on 2048^2, 35 of them HBM's;
+// bound by its instructions (IEEE divisions and square roots; whole waves of
+// taller segments 54.5 us, a row of prefetch 60, shuffles for the ring 55.5).
 constexpr int FIELD_T = 128, FIELD_COLS = FIELD_T - 2, FIELD_ROWS = 16;
 
 __global__ void __launch_bounds__(FIELD_T) fields_kernel(const StepParams P, float* __restrict__ orho,
@@ -224,7 +226,7 @@ struct Parts {
 // Sum of f over the cells and directions, exact up to the FP64 sum of runs of
 // 64 values. Warps take rows of the nine planes, four columns per lane and
 // load. FP64 adds run at 1/64 of the FP32 rate: one per value took 154 us on
-// 2048^2 (22 us from HBM), one per run of 64 takes the figure of the read.
+// 2048^2 (22 us from HBM), one per run of 64 takes 28.
 __global__ void __launch_bounds__(256) mass_kernel(const StepParams P, const float* __restrict__ f) {
     __shared__ double red[8];
     double t = 0.0;
