@@ -195,8 +195,8 @@ __device__ __forceinline__ void rev_coef_vals(const StepParams& P, const AdjFiel
 // second in the next iteration. Walls in y only (the adjoint's supported
 // case).
 //
-// What bounds it: the shared-memory path and fixed-latency waits at twelve
-// warps per SM (165 registers). 2048^2: 83 us per launch, 105 us for one row
+// What bounds it: the issue slots (62 %) and the L1 and shared-memory path
+// (61 %) at twelve warps per SM (165 registers); HBM is 42 % busy. 2048^2: 83 us per launch, 105 us for one row
 // per iteration with nine-point sums (20 warps); 69 bytes per cell, 43 us from
 // HBM. Held to 128 registers (16 warps, 120 bytes of spill) it takes as long as
 // that; blocks of 64 and 192 threads are 1-2 us slower, of 256 17 us; loading
