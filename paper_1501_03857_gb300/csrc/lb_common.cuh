@@ -28,10 +28,12 @@ struct Cols {
 // Pulled populations (Eq. 3: f_a(x) = f*_a(x - e_a)) and theta of row y for
 // the two columns. S: rows y - 1 .. y + 1 lie inside. Otherwise the source
 // rows are clamped to the domain (the outflow top's zero-gradient condition;
-// on wall rows the Zou-He fill replaces what was pulled from there).
-template <bool CG, bool S>
+// on wall rows the Zou-He fill replaces what was pulled from there). Coherent
+// loads (lb_ldco): the step before, still running when this kernel starts,
+// writes these planes.
+template <bool S>
 __device__ __forceinline__ void load_row2(const StepParams& P, int y, const Cols& c, P2 (&f)[9], P2& th) {
-    const float* __restrict__ F = P.f_in;
+    const float* F = P.f_in;
     const int pl = P.plane, pitch = P.pitch;
     const size_t nF = 9 * (size_t)pl;
     int ym = y - 1, yp = y + 1;
@@ -46,7 +48,7 @@ __device__ __forceinline__ void load_row2(const StepParams& P, int y, const Cols
     }
     auto ld = [&](int a, int row, int xa, int xb) {
         const int o = a * pl + row * pitch;
-        return P2(lb_ld<CG>(F + (o + xa), F, nF, P.acc), lb_ld<CG>(F + (o + xb), F, nF, P.acc));
+        return P2(lb_ldco(F + (o + xa), F, nF, P.acc), lb_ldco(F + (o + xb), F, nF, P.acc));
     };
     f[0] = ld(0, y, c.a, c.b);
     f[1] = ld(1, y, c.am, c.bm);
@@ -58,7 +60,7 @@ __device__ __forceinline__ void load_row2(const StepParams& P, int y, const Cols
     f[7] = ld(7, yp, c.ap, c.bp);
     f[8] = ld(8, yp, c.am, c.bm);
     const int o = y * pitch;
-    th = P2(lb_ld<CG>(P.th_in + (o + c.a), P.th_in, (size_t)pl, P.acc), lb_ld<CG>(P.th_in + (o + c.b), P.th_in, (size_t)pl, P.acc));
+    th = P2(lb_ldco(P.th_in + (o + c.a), P.th_in, (size_t)pl, P.acc), lb_ldco(P.th_in + (o + c.b), P.th_in, (size_t)pl, P.acc));
 }
 
 __device__ __forceinline__ P2 sel(bool c, P2 a, P2 b) { return P2(c ? a.x() : b.x(), c ? a.y() : b.y()); }

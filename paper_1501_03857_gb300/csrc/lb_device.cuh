@@ -92,6 +92,11 @@ __device__ __forceinline__ bool finite_f(float v) { return fabsf(v) <= 3.4028234
 // shared-memory access of the fused step goes through these; an address
 // outside its buffer sets ERR_BOUNDS and the access is skipped (a load reads
 // 0) instead of faulting. In the normal build they are the plain accesses.
+// Loads of the state, which another grid or block writes while this kernel
+// runs (kernels overlap their predecessor, grid_start; the persistent batch's
+// blocks exchange buffers), are plain coherent ones (lb_ldco): after the wait
+// they see those writes, where the read-only path (lb_ldg, for the wall
+// temperature, which only copies write) may serve data it cached before.
 #ifdef LB_CHECKED
 __device__ __forceinline__ bool lb_inside(const void* p, const void* base, size_t bytes, size_t width, Acc* acc) {
     const char* c = static_cast<const char*>(p);
@@ -124,17 +129,6 @@ __device__ __forceinline__ void lb_st_if(bool on, float* p, float v, const float
     asm volatile("{ .reg .pred q; setp.ne.u32 q, %2, 0; @q st.global.f32 [%0], %1; }" ::"l"(p), "f"(v), "r"((unsigned)on));
 #endif
 }
-// Loads of the step's input state: through the read-only path in a kernel
-// that runs one step (lb_ldg), as plain coherent loads (lb_ldco) in the
-// persistent batch, where other blocks rewrite the buffers during the launch:
-// the read-only path may serve data it cached before that; a plain load after
-// the block's acquire of the other blocks' progress sees their writes.
-template <bool CO>
-__device__ __forceinline__ float lb_ld(const float* p, const float* base, size_t n, Acc* acc) {
-    if constexpr (CO) return lb_ldco(p, base, n, acc);
-    else return lb_ldg(p, base, n, acc);
-}
-
 // psi(rho, T) = sqrt(2 (p_EOS - rho c_s^2) / G), c = 1 (Sec. 2 and Eq. 21).
 __device__ __forceinline__ float eos_psi(float rho, float T, const StepParams& P, bool& bad) {
     const float sT = sqrtf(T);

@@ -14,10 +14,10 @@ template <int MINB>
 struct MarchFormT {
     static constexpr int threads = MARCH_T, min_blocks = MINB;
     static constexpr int smem = MarchSmem::total * (int)sizeof(float2);
-    template <bool REC, bool CG, bool OUT, bool QF>
+    template <bool REC, bool OUT, bool QF>
     static __device__ __forceinline__ void body(const StepParams& P, const StepParams& C, int block, int fold,
                                                 const RecomputeOut* R) {
-        march_body<REC, CG, OUT, QF>(P, C, block, fold, R);
+        march_body<REC, OUT, QF>(P, C, block, fold, R);
     }
 };
 
@@ -31,10 +31,10 @@ template <int NW, int K>
 struct TileForm {
     static constexpr int threads = NW * 32, min_blocks = 1;
     static constexpr int smem = TileShape<NW, K>::slots * (int)sizeof(float2);
-    template <bool REC, bool CG, bool OUT, bool QF>
+    template <bool REC, bool OUT, bool QF>
     static __device__ __forceinline__ void body(const StepParams& P, const StepParams& C, int block, int fold,
                                                 const RecomputeOut* R) {
-        tile_body<NW, K, REC, CG, OUT, QF>(P, C, block, fold, R);
+        tile_body<NW, K, REC, OUT, QF>(P, C, block, fold, R);
     }
 };
 using Tile24 = TileForm<12, 2>;

@@ -54,7 +54,7 @@ struct MarchSmem {
 // The whole step for block `block`: column pair block % npair, segment of
 // P.seg_h rows. C supplies the model constants (see lb_step_batch.cu); fold: the
 // previous step's q(t) is still to be folded.
-template <bool REC, bool CG, bool OUT, bool QF>
+template <bool REC, bool OUT, bool QF>
 __device__ __forceinline__ void march_body(const StepParams& P, const StepParams& C, const int block, const int fold,
                                            const RecomputeOut* R) {
     extern __shared__ float2 sm2[];
@@ -115,8 +115,8 @@ __device__ __forceinline__ void march_body(const StepParams& P, const StepParams
 #pragma unroll
     for (int a = 0; a < 9; ++a) fp[a] = zero;
     const int L0 = periodic ? ys - HALO : max(ys - HALO, 0);
-    load_row2<CG, false>(P, phys(L0), c, f0, th0);
-    load_row2<CG, false>(P, phys(L0 + 1), c, f1, th1);
+    load_row2<false>(P, phys(L0), c, f0, th0);
+    load_row2<false>(P, phys(L0 + 1), c, f1, th1);
     // own values of the previous half's rows
     P2 cpsi0 = zero, cpsi1 = zero, cvx = zero, cvy0 = zero, cvy1 = zero, crho0 = zero, crho1 = zero;
     P2 cu20 = zero, cu21 = zero, cu30 = zero, cu31 = zero, cu40 = zero, cu41 = zero;
@@ -233,8 +233,8 @@ __device__ __forceinline__ void march_body(const StepParams& P, const StepParams
         for (int a = 0; a < 9; ++a) fp[a] = f1[a];
         rhop = rho1;
         if (S || L + 2 < ye + HALO) {
-            load_row2<CG, S>(P, S ? L + 2 : phys(L + 2), c, f0, th0);
-            load_row2<CG, S>(P, S ? L + 3 : phys(L + 3), c, f1, th1);
+            load_row2<S>(P, S ? L + 2 : phys(L + 2), c, f0, th0);
+            load_row2<S>(P, S ? L + 3 : phys(L + 3), c, f1, th1);
         }
         __syncthreads();
 

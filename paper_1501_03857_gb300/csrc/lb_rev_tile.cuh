@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(NW * 32) rev_tile(const StepParams P, AdjField
         return Row3{P2(q[-1]), P2(q[0]), P2(q[1])};
     };
     auto cell = [&](int F, int k) { return P2(*at(own + F * Sh::field + k * TILE_ROW)); };
-    auto load = [&](const float* __restrict__ p, int r) {  // (rows beyond the wall: the wall row's value)
+    auto load = [&](const float* p, int r) {  // (rows beyond the wall: the wall row's value)
         const int i = min(r, Ly - 1) * pitch;
         return P2(LB_LD(p, i + c.a, pl), LB_LD(p, i + c.b, pl));
     };
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(NW * 32) rev_tile(const StepParams P, AdjField
             if (isrow(y) && y + 1 >= ys && y < ye + 1) {
                 const bool wall = wallrow(y);
                 P2 f[9], lo[9], t;
-                load_row2<false, false>(P, y, c, f, t);
+                load_row2<false>(P, y, c, f, t);
 #pragma unroll
                 for (int a = 0; a < 9; ++a)
                     lo[a] = P2(LB_LD(A.lf_in, a * pl + y * pitch + c.a, 9 * (size_t)pl),

@@ -13,7 +13,7 @@ namespace {
 template <class F>
 __global__ void __launch_bounds__(F::threads, F::min_blocks) lb_step_kernel(const StepParams P, const int fold) {
     grid_start();
-    F::template body<false, false, true, true>(P, P, blockIdx.x, fold, nullptr);
+    F::template body<false, true, true>(P, P, blockIdx.x, fold, nullptr);
 }
 
 // q(t) of the last step of a call (fold_heat): one warp.

@@ -34,7 +34,7 @@ __global__ void __launch_bounds__(F::threads, F::min_blocks)
     copy_params<F::threads>(table + tl.x, sP);
     __syncthreads();
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    F::template body<false, false, true, true>(sP, SK ? K : sP, tl.y, fold, nullptr);
+    F::template body<false, true, true>(sP, SK ? K : sP, tl.y, fold, nullptr);
 }
 
 // q(t) of every instance's last step of a call: one warp per instance, from
@@ -57,11 +57,10 @@ __global__ void __launch_bounds__(32) lb_batch_fold(const StepParams* __restrict
 // zero at launch). A wait polls the root at most `wait_limit` times; a block
 // that gives up sets ERR_TIMEOUT in its first instance's fault flags and
 // leaves the kernel, which lets every block waiting on it give up in turn, so
-// the launch always ends. The step's input state is read with plain loads,
-// which after the acquiring fence and the block's barrier see the other SMs'
-// writes (the read-only path could serve copies cached before them), and every
-// tile runs the same step as the per-step kernel, so results are bit-identical
-// to it.
+// the launch always ends. The step's loads of its input state are coherent
+// (lb_ldco), so after the acquiring fence and the block's barrier they see the
+// other SMs' writes; every tile runs the same step as the per-step kernel, so
+// results are bit-identical to it.
 //
 // Waiting only for the tile's own instance, as this kernel did before, lets
 // the instances drift apart, and blocks at different stages of their march
@@ -103,7 +102,7 @@ __global__ void __launch_bounds__(F::threads, F::min_blocks) lb_batch_persist(co
                 copy_params<BD>(A.table + (k & 1) * A.n + tl.x, sP);
                 __syncthreads();
             }
-            F::template body<false, true, true, true>(sP, SK ? K : sP, tl.y, k > 0, nullptr);
+            F::template body<false, true, true>(sP, SK ? K : sP, tl.y, k > 0, nullptr);
             __syncthreads();
         }
         if (threadIdx.x == 0) {

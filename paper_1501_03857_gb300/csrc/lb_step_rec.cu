@@ -11,7 +11,7 @@ template <class F, bool OUT, bool QF>
 __global__ void __launch_bounds__(F::threads, F::min_blocks)
     lb_step_recompute(const StepParams P, const __grid_constant__ RecomputeOut R, const int fold) {
     grid_start();
-    F::template body<true, false, OUT, QF>(P, P, blockIdx.x, fold, &R);
+    F::template body<true, OUT, QF>(P, P, blockIdx.x, fold, &R);
 }
 
 template <class F, bool OUT, bool QF>

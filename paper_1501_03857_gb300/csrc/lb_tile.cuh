@@ -43,7 +43,7 @@ struct TileShape {
 };
 
 // Output rows [ys, ye) and columns [x0, x0 + nv) of the step.
-template <int NW, int K, bool REC, bool CG, bool OUT, bool QF>
+template <int NW, int K, bool REC, bool OUT, bool QF>
 __device__ __forceinline__ void tile_rows(const StepParams& P, const StepParams& C, int x0, int nv, int ys, int ye,
                                           const RecomputeOut* R, float2* sm, bool& eos_bad, bool& nonfinite) {
     using Sh = TileShape<NW, K>;
@@ -109,7 +109,7 @@ __device__ __forceinline__ void tile_rows(const StepParams& P, const StepParams&
     P2 f[K][9], rho[K], th[K];
     if (any(HALO)) {
 #pragma unroll
-        for (int k = 0; k < K; ++k) load_row2<CG, false>(P, phys(r0 + k), c, f[k], th[k]);
+        for (int k = 0; k < K; ++k) load_row2<false>(P, phys(r0 + k), c, f[k], th[k]);
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const int y = r0 + k;
@@ -338,7 +338,7 @@ __device__ __forceinline__ void tile_rows(const StepParams& P, const StepParams&
 // The whole step for block `block`: strip block % nstrips, and the rows of its
 // segment (P.seg_h, normally one tile's). K = C supplies the model constants
 // (see lb_step_batch.cu); fold: the previous step's q(t) is still to be folded.
-template <int NW, int K, bool REC, bool CG, bool OUT, bool QF>
+template <int NW, int K, bool REC, bool OUT, bool QF>
 __device__ __forceinline__ void tile_body(const StepParams& P, const StepParams& C, const int block, const int fold,
                                           const RecomputeOut* R) {
     extern __shared__ float2 sm2[];
@@ -351,7 +351,7 @@ __device__ __forceinline__ void tile_body(const StepParams& P, const StepParams&
     const int s1 = min((seg + 1) * P.seg_h, P.Ly);
     for (int ys = seg * P.seg_h; ys < s1; ys += Sh::out) {
         if (ys > seg * P.seg_h) __syncthreads();
-        tile_rows<NW, K, REC, CG, OUT, QF>(P, C, x0, nv, ys, min(ys + Sh::out, s1), R, sm2, eos_bad, nonfinite);
+        tile_rows<NW, K, REC, OUT, QF>(P, C, x0, nv, ys, min(ys + Sh::out, s1), R, sm2, eos_bad, nonfinite);
     }
     if (eos_bad) atomicOr(&P.acc->err, ERR_EOS);
     if (nonfinite) atomicOr(&P.acc->err, ERR_NONFINITE);
