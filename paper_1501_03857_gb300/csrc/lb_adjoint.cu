@@ -904,12 +904,30 @@ cudaError_t adjoint_grads_finish(const StepParams& P, void* work, const float* l
     return e;
 }
 
+cudaError_t adjoint_prepare(ReverseShape* S) {
+    ReverseShape r{};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&r.nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = allow_smem((const void*)rev_thermal_fused, (int)rt_smem_bytes());
+    if (e == cudaSuccess) e = allow_smem((const void*)rev_tile<RV_NW, RV_K>, RV_SMEM);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r.occ_t, rev_thermal_fused, RT_BD, rt_smem_bytes());
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r.occ_f, rev_flow_fused, RF_BD, 0);
+    if (e != cudaSuccess) return e;
+    r.occ_t = std::max(r.occ_t, 1);
+    r.occ_f = std::max(r.occ_f, 1);
+    *S = r;
+    return cudaSuccess;
+}
+
 // One reverse step: state (fstar, theta) of level n and the intermediates R
 // of the step from it, lambda of level n+1 in (lf_in with lr_in, lt_in),
 // lambda of level n out (lf_out with lr_out, lt_out); lq = dJ/dq(t_n).
-cudaError_t adjoint_reverse_step(const StepParams& P, const RecomputeOut& R, void* work, const float* fstar,
-                                 const float* theta, const float* lf_in, const float* lt_in, const float* lr_in,
-                                 float* lf_out, float* lt_out, float* lr_out, float lq, cudaStream_t st) {
+cudaError_t adjoint_reverse_step(const ReverseShape& S, const StepParams& P, const RecomputeOut& R, void* work,
+                                 const float* fstar, const float* theta, const float* lf_in, const float* lt_in,
+                                 const float* lr_in, float* lf_out, float* lt_out, float* lr_out, float lq,
+                                 cudaStream_t st) {
     AdjFields A = fields_at(P, work);
     A.fstar = fstar;
     A.theta = theta;
@@ -932,31 +950,7 @@ cudaError_t adjoint_reverse_step(const StepParams& P, const RecomputeOut& R, voi
     // the four RK stages transposed, then the collision, forces, psi and the
     // pull: two column-marching launches, segments sized so that the blocks
     // fill the GPU once
-    // SM count and blocks per SM of the two reverse kernels: looked up once
-    // (a function-local static: initialised once, also under concurrent
-    // first calls)
-    struct RevShape {
-        cudaError_t e;
-        int nsm, occ_t, occ_f;
-    };
-    static const RevShape RS = [] {
-        RevShape r{cudaSuccess, 0, 0, 0};
-        int dev = 0;
-        r.e = cudaGetDevice(&dev);
-        if (r.e == cudaSuccess) r.e = cudaDeviceGetAttribute(&r.nsm, cudaDevAttrMultiProcessorCount, dev);
-        if (r.e == cudaSuccess)
-            r.e = cudaFuncSetAttribute(rev_thermal_fused, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)rt_smem_bytes());
-        if (r.e == cudaSuccess)
-            r.e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r.occ_t, rev_thermal_fused, RT_BD, rt_smem_bytes());
-        if (r.e == cudaSuccess) r.e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r.occ_f, rev_flow_fused, RF_BD, 0);
-        if (r.e == cudaSuccess) r.e = allow_smem((const void*)rev_tile<RV_NW, RV_K>, RV_SMEM);
-        r.occ_t = std::max(r.occ_t, 1);
-        r.occ_f = std::max(r.occ_f, 1);
-        return r;
-    }();
-    if (RS.e != cudaSuccess) return RS.e;
-    const int nsm = RS.nsm, occ_t = RS.occ_t, occ_f = RS.occ_f;
+    const int nsm = S.nsm, occ_t = S.occ_t, occ_f = S.occ_f;
     const int tiles = (P.Lx + RV_COLS - 1) / RV_COLS * rev_tiles<RevShape2<RV_NW, RV_K>>(P.Ly);
     // the tiles while they come to one wave (one block per SM, 13 us; a step of
     // the whole adjoint, us, tiles against marching: 600 x 150 28.8 and 34.6,

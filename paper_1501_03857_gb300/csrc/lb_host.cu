@@ -222,6 +222,7 @@ struct lb_handle {
     cudaEvent_t adj_in, adj_out;
     cudaStream_t adj_stream2;           // recompute stream of the adjoint
     cudaEvent_t adj_ready[2], adj_free[2];  // segment buffer filled / released
+    ReverseShape rev;                       // nsm 0 until the first adjoint
     struct AdjGraph {
         int kind;  // 0: recompute into a segment buffer, 1: reverse sweep over it
         int len, cur, buf, C, nsteps;
@@ -642,6 +643,7 @@ int lb_init(lb_handle** out, const lb_grid* grid, const lb_eos* eos, const lb_th
     h->adj_in = h->adj_out = nullptr;
     h->adj_stream2 = nullptr;
     h->adj_ready[0] = h->adj_ready[1] = h->adj_free[0] = h->adj_free[1] = nullptr;
+    h->rev = ReverseShape{};
     {
         cudaError_t e0 = cudaMallocHost((void**)&h->rec, sizeof(Acc) + grid->Lx * sizeof(float));
         if (e0 == cudaSuccess) h->wall_pinned = (float*)(h->rec + 1);
@@ -1654,6 +1656,8 @@ int lb_adjoint(lb_handle* h, int nsteps, int ckpt_every, void* dev_scratch, size
     if (!dev_scratch || scratch_bytes < L.total)
         return fail(LB_E_INVAL, "adjoint scratch of %zu bytes is smaller than the %zu needed", scratch_bytes, L.total);
     if (((uintptr_t)dev_scratch) & 255) return fail(LB_E_INVAL, "scratch must be 256-byte aligned");
+    // per handle: a function's shared-memory limit belongs to the device
+    if (h->rev.nsm == 0) LB_CUDA(adjoint_prepare(&h->rev), "reverse kernels");
     char* s = (char*)dev_scratch;
     const size_t pl = (size_t)base.plane;
     const size_t state = align256(sizeof(float) * 10 * pl);
@@ -1775,8 +1779,9 @@ int lb_adjoint(lb_handle* h, int nsteps, int ckpt_every, void* dev_scratch, size
         int c = c0;
         for (int j = len - 1; j >= 0; --j) {
             const float* fs = seg_state(buf, j);
-            LB_CUDA(adjoint_reverse_step(RB, seg_rec(buf, j), work, fs, fs + 9 * pl, lam[c], lam[c] + 9 * pl,
-                                         lam[c] + 10 * pl, lam[1 - c], lam[1 - c] + 9 * pl, lam[1 - c] + 10 * pl, lq, q),
+            LB_CUDA(adjoint_reverse_step(h->rev, RB, seg_rec(buf, j), work, fs, fs + 9 * pl, lam[c],
+                                         lam[c] + 9 * pl, lam[c] + 10 * pl, lam[1 - c], lam[1 - c] + 9 * pl,
+                                         lam[1 - c] + 10 * pl, lq, q),
                     "adjoint reverse step");
             c ^= 1;
         }
@@ -1787,8 +1792,9 @@ int lb_adjoint(lb_handle* h, int nsteps, int ckpt_every, void* dev_scratch, size
     auto sweep_all = [&](cudaStream_t q) -> int {
         int c = 0;
         for (int j = nsteps - 1; j >= 0; --j) {
-            LB_CUDA(adjoint_reverse_step(RB, rec_at((size_t)j), work, state_f(j), state_t(j), lam[c], lam[c] + 9 * pl,
-                                         lam[c] + 10 * pl, lam[1 - c], lam[1 - c] + 9 * pl, lam[1 - c] + 10 * pl, lq, q),
+            LB_CUDA(adjoint_reverse_step(h->rev, RB, rec_at((size_t)j), work, state_f(j), state_t(j), lam[c],
+                                         lam[c] + 9 * pl, lam[c] + 10 * pl, lam[1 - c], lam[1 - c] + 9 * pl,
+                                         lam[1 - c] + 10 * pl, lq, q),
                     "adjoint reverse step");
             c ^= 1;
         }

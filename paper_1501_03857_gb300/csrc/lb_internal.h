@@ -90,9 +90,15 @@ cudaError_t launch_fields(const StepParams& P, float* rho, float* ux, float* uy,
 cudaError_t launch_macro(const StepParams& P, float* scratch, float* rho, float* ux, float* uy,
                          float* T, int ostride, cudaStream_t st);
 
-// Discrete adjoint of one step (lb_adjoint.cu): work bytes, reset of the
-// FP64 gradient accumulators, one reverse step, and the final read-out
-// (which adds the initial wall row's lambda_theta to dJ/d theta_b).
+// Discrete adjoint of one step (lb_adjoint.cu): what the current device gives
+// the reverse kernels (SMs, blocks per SM), opting them in to their dynamic
+// shared memory there; work bytes, reset of the FP64 gradient accumulators,
+// one reverse step, and the final read-out (which adds the initial wall row's
+// lambda_theta to dJ/d theta_b).
+struct ReverseShape {
+    int nsm, occ_t, occ_f;
+};
+cudaError_t adjoint_prepare(ReverseShape* S);
 size_t adjoint_work_bytes(const StepParams& P);
 cudaError_t adjoint_grads_reset(const StepParams& P, void* work, cudaStream_t st);
 // The adjoint of f* travels between reverse steps in two parts: lambda of
@@ -102,9 +108,10 @@ cudaError_t adjoint_grads_reset(const StepParams& P, void* work, cudaStream_t st
 // and lr are a zero adjoint. The in and out planes are distinct buffers.
 // R holds the forward intermediates of the step being reversed (written by
 // launch_recompute from the same state).
-cudaError_t adjoint_reverse_step(const StepParams& P, const RecomputeOut& R, void* work, const float* fstar,
-                                 const float* theta, const float* lf_in, const float* lt_in, const float* lr_in,
-                                 float* lf_out, float* lt_out, float* lr_out, float lq, cudaStream_t st);
+cudaError_t adjoint_reverse_step(const ReverseShape& S, const StepParams& P, const RecomputeOut& R, void* work,
+                                 const float* fstar, const float* theta, const float* lf_in, const float* lt_in,
+                                 const float* lr_in, float* lf_out, float* lt_out, float* lr_out, float lq,
+                                 cudaStream_t st);
 cudaError_t adjoint_grads_finish(const StepParams& P, void* work, const float* lt0, double* dTb_host,
                                  double* dGw_host, cudaStream_t st);
 

@@ -53,3 +53,11 @@ def test_overlapped_kernels_read_written_data_coherently():
             if "__restrict__" in line:
                 assert re.search(r"const (StepParams|int2)\* __restrict__ (src|table|tiles)\b", line), (name, line)
                 assert "float" not in line.split("__restrict__")[0], (name, line)
+
+
+def test_nothing_about_a_device_is_kept_for_the_process():
+    """A shared-memory opt-in, an SM count or an occupancy looked up once per
+    process would serve a second device's launches with the first one's."""
+    for path in glob.glob(os.path.join(CSRC, "*.[ch]*")):
+        for line in source(os.path.basename(path)).splitlines():
+            assert not re.match(r"\s+(static|thread_local)\s+(?!constexpr|__device__)[^()]*=", line), (path, line)
