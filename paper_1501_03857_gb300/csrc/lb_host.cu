@@ -209,6 +209,7 @@ struct lb_handle {
     double* qpart;
     int cur;
     cudaStream_t st;
+    int dev;                 // the device the workspace is on
     int64_t steps;
     Launch launch;
     StepParams base;
@@ -410,10 +411,26 @@ int report_device_errors(lb_handle* h, unsigned err) {
     return LB_OK;
 }
 
+// Makes a device current while it lives. The read-backs and state copies are
+// kernels, which run on the current device, where copies run wherever their
+// memory is: a caller may have another device current.
+struct OnDevice {
+    int before = -1;
+    explicit OnDevice(int dev) {
+        if (cudaGetDevice(&before) != cudaSuccess || before == dev || cudaSetDevice(dev) != cudaSuccess) before = -1;
+    }
+    ~OnDevice() {
+        if (before >= 0) cudaSetDevice(before);
+    }
+    OnDevice(const OnDevice&) = delete;
+    OnDevice& operator=(const OnDevice&) = delete;
+};
+
 // The accumulator record into h->rec, after everything issued on the stream:
 // one launch that writes pinned memory and one wait (a read into pageable
 // memory waits once more); reset clears the heat-flux sums.
 int read_acc(lb_handle* h, bool reset = false) {
+    const OnDevice on(h->dev);
     LB_CUDA(launch_collect(nullptr, h->acc, 1, h->rec, reset, h->st), "read accumulators");
     LB_CUDA(cudaStreamSynchronize(h->st), "cudaStreamSynchronize");
     return LB_OK;
@@ -424,12 +441,11 @@ int check_device_errors(lb_handle* h) {
     return rc ? rc : report_device_errors(h, h->rec->err);
 }
 
-// Whether p is float-aligned memory of the current device (else copies go
-// through cudaMemcpy, which takes any address).
-bool on_this_device(const void* p) {
+// Whether p is float-aligned memory of device dev (else copies go through
+// cudaMemcpy, which takes any address).
+bool on_device_memory(const void* p, int dev) {
     cudaPointerAttributes a;
-    int dev = -1;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
@@ -634,6 +650,7 @@ int lb_init(lb_handle** out, const lb_grid* grid, const lb_eos* eos, const lb_th
     h->qpart = (double*)(h->ws + lay.qpart);
     h->cur = 0;
     h->st = (cudaStream_t)stream;
+    h->dev = 0;
     h->steps = 0;
     h->rec = nullptr;
     h->wall_pinned = nullptr;
@@ -645,7 +662,8 @@ int lb_init(lb_handle** out, const lb_grid* grid, const lb_eos* eos, const lb_th
     h->adj_ready[0] = h->adj_ready[1] = h->adj_free[0] = h->adj_free[1] = nullptr;
     h->rev = ReverseShape{};
     {
-        cudaError_t e0 = cudaMallocHost((void**)&h->rec, sizeof(Acc) + grid->Lx * sizeof(float));
+        cudaError_t e0 = cudaGetDevice(&h->dev);
+        if (e0 == cudaSuccess) e0 = cudaMallocHost((void**)&h->rec, sizeof(Acc) + grid->Lx * sizeof(float));
         if (e0 == cudaSuccess) h->wall_pinned = (float*)(h->rec + 1);
         if (e0 == cudaSuccess) e0 = cudaEventCreateWithFlags(&h->wall_done, cudaEventDisableTiming);
         if (e0 != cudaSuccess) {
@@ -773,7 +791,9 @@ int lb_get_state(lb_handle* h, float* fpost, float* theta, int on_device) {
     if (!h) return fail(LB_E_INVAL, "null handle");
     const int Lx = h->grid.Lx, Ly = h->grid.Ly, pitch = h->lay.pitch;
     const cudaMemcpyKind k = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-    if (on_device && (fpost || theta) && (!fpost || on_this_device(fpost)) && (!theta || on_this_device(theta))) {
+    if (on_device && (fpost || theta) && (!fpost || on_device_memory(fpost, h->dev)) &&
+        (!theta || on_device_memory(theta, h->dev))) {
+        const OnDevice on(h->dev);
         LB_CUDA(launch_copy_state(fpost ? h->f[h->cur] : nullptr, fpost, theta ? h->t[h->cur] : nullptr, theta, Lx, Ly,
                                   pitch, Lx, &h->acc->err, &h->rec->err, h->st),
                 "state copy");
@@ -795,7 +815,9 @@ int lb_set_state(lb_handle* h, const float* fpost, const float* theta, int on_de
     if (!h) return fail(LB_E_INVAL, "null handle");
     const int Lx = h->grid.Lx, Ly = h->grid.Ly, pitch = h->lay.pitch;
     const cudaMemcpyKind k = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    if (on_device && (fpost || theta) && (!fpost || on_this_device(fpost)) && (!theta || on_this_device(theta))) {
+    if (on_device && (fpost || theta) && (!fpost || on_device_memory(fpost, h->dev)) &&
+        (!theta || on_device_memory(theta, h->dev))) {
+        const OnDevice on(h->dev);
         LB_CUDA(launch_copy_state(fpost, h->f[h->cur], theta, h->t[h->cur], Lx, Ly, Lx, pitch, nullptr, nullptr, h->st),
                 "state copy");
         return LB_OK;
@@ -1497,6 +1519,7 @@ int lb_batch_step(lb_batch* b, int nsteps) {
 static int batch_read(lb_batch* b, bool reset) {
     int rc = batch_upload(b);  // the table names the instances' records
     if (rc) return rc;
+    const OnDevice on(b->inst[0]->dev);
     LB_CUDA(launch_collect(b->table, nullptr, (int)b->inst.size(), b->rec, reset, b->st), "read accumulators");
     LB_CUDA(cudaStreamSynchronize(b->st), "cudaStreamSynchronize");
     int first = LB_OK;

@@ -61,3 +61,17 @@ def test_nothing_about_a_device_is_kept_for_the_process():
     for path in glob.glob(os.path.join(CSRC, "*.[ch]*")):
         for line in source(os.path.basename(path)).splitlines():
             assert not re.match(r"\s+(static|thread_local)\s+(?!constexpr|__device__)[^()]*=", line), (path, line)
+
+
+def test_read_backs_run_on_their_own_device():
+    """Read-backs and state copies were copies, which run wherever their
+    memory is; as kernels they need their handle's device to be current."""
+    text = source("lb_host.cu")
+    seen = 0
+    for m in re.finditer(r"\b(launch_collect|launch_copy_state)\(", text):
+        scope = text.rfind("const OnDevice on(", 0, m.start())
+        assert scope >= 0 and "\n}\n" not in text[scope:m.start()], text[m.start() - 200:m.start() + 40]
+        seen += 1
+    assert seen == 4
+    asked = [args for _, args in calls(text, "on_device_memory") if not args.startswith("const void*")]
+    assert len(asked) == 4 and all(a.endswith("h->dev") for a in asked)
