@@ -285,6 +285,17 @@ cudaError_t launch_macro(const StepParams& P, float* scratch, float* rho, float*
     return cudaGetLastError();
 }
 
+// A launch that returns its own status: cudaGetLastError after it would also
+// report an earlier call's failure, which these read-backs may follow.
+template <class... A, class... B>
+static cudaError_t launch(void (*kernel)(A...), int blocks, int threads, cudaStream_t st, B... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = st;
+    return cudaLaunchKernelEx(&cfg, kernel, A(args)...);
+}
+
 cudaError_t launch_copy_state(const float* f_src, float* f_dst, const float* t_src, float* t_dst, int Lx, int Ly,
                               int src_pitch, int dst_pitch, const unsigned* err, unsigned* err_out,
                               cudaStream_t st) {
@@ -294,11 +305,8 @@ cudaError_t launch_copy_state(const float* f_src, float* f_dst, const float* t_s
     const int blocks = (int)std::min<long long>((warps + 7) / 8, 16 * 152);
     if (blocks == 0) return cudaSuccess;
     // (the pitch is a multiple of 32 floats: the other side's rows decide)
-    if (all % 16 == 0 && Lx % 4 == 0)
-        copy_rows<4><<<blocks, 256, 0, st>>>(f_src, f_dst, n0, t_src, t_dst, n1, Lx, src_pitch, dst_pitch, err, err_out);
-    else
-        copy_rows<1><<<blocks, 256, 0, st>>>(f_src, f_dst, n0, t_src, t_dst, n1, Lx, src_pitch, dst_pitch, err, err_out);
-    return cudaGetLastError();
+    auto kernel = all % 16 == 0 && Lx % 4 == 0 ? copy_rows<4> : copy_rows<1>;
+    return launch(kernel, blocks, 256, st, f_src, f_dst, n0, t_src, t_dst, n1, Lx, src_pitch, dst_pitch, err, err_out);
 }
 
 // The accumulator records of a batch's instances (table) or of one simulation
@@ -313,8 +321,7 @@ __global__ void collect_acc(const StepParams* __restrict__ table, Acc* acc, int 
 }
 
 cudaError_t launch_collect(const StepParams* table, Acc* acc, int n, Acc* out, bool reset, cudaStream_t st) {
-    collect_acc<<<(n + 63) / 64, 64, 0, st>>>(table, acc, n, out, reset ? 1 : 0);
-    return cudaGetLastError();
+    return launch(collect_acc, (n + 63) / 64, 64, st, table, acc, n, out, reset ? 1 : 0);
 }
 
 cudaError_t launch_fields(const StepParams& P, float* rho, float* ux, float* uy, float* T, int ostride,
