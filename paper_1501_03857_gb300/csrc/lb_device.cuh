@@ -59,25 +59,30 @@ struct StepParams {
     // the constants of the paired FP32 arithmetic, each duplicated into a
     // float2 so that a paired instruction can take it from the parameter
     // bank as it is (set_pairs)
-    float2 kp[27];
+    float2 kp[28];
 };
 
 enum {
     KP_TS, KP_K1N, KP_K0, KP_B, KP_R, KP_A, KP_2G, KP_K0K1N, KP_K1K1, KP_CHI6,
     KP_SE36N, KP_KE6, KP_KESIG, KP_SZ12N, KP_KZ6N, KP_KZSIGN, KP_SQ6, KP_SQ12N, KP_DTAU4, KP_TAUV4,
-    KP_GN12, KP_GW6, KP_GN, KP_RHOAVE, KP_CHI144, KP_RCV12, KP_ACV12, KP_COUNT
+    KP_GN12, KP_GW6, KP_GN, KP_RHOAVE, KP_CHI144, KP_RCV12, KP_ACV12, KP_PSI, KP_COUNT
 };
 
 // Fill kp from the scalar fields (after any of them changes).
 inline void set_pairs(StepParams& P) {
     static_assert(KP_COUNT == sizeof(P.kp) / sizeof(P.kp[0]), "kp size");
     const float G2 = P.G * P.G * (1.f / 144.f);
+    // psi^2 is formed times 4^k, with |2 / G| 4^k in [2^54, 2^56): the smallest
+    // |p - rho/3|, 2^-149, then gives at least 2^-95, and only beyond 2^72 does
+    // it overflow
+    const float tg = fabsf(P.two_over_G);
+    const int k = tg > 0.f && tg <= 3.402823466e38f ? (55 - ilogbf(tg)) >> 1 : 0;
     const float ke = (1.f - 0.5f * P.s_e) * (1.f / 36.f), kz = (1.f - 0.5f * P.s_z) * (1.f / 36.f);
-    const float v[KP_COUNT] = {P.Ts, -P.k1, P.k0, P.b, P.R, P.a, P.two_over_G, -P.k0k1, P.k1k1, P.chi * (1.f / 6.f),
+    const float v[KP_COUNT] = {P.Ts, -P.k1, P.k0, P.b, P.R, P.a, ldexpf(P.two_over_G, 2 * k), -P.k0k1, P.k1k1, P.chi * (1.f / 6.f),
                                -P.s_e * (1.f / 36.f), 6.f * ke, ke * P.sig_e * G2, -P.s_z * (1.f / 12.f), -6.f * kz,
                                -kz * P.sig_z * G2, P.s_q * (1.f / 6.f), -P.s_q * (1.f / 12.f), 4.f * P.dtau,
                                4.f * P.tau_v, -P.G * (1.f / 12.f), P.gw6, -P.g, P.rho_ave, P.chi * (1.f / 144.f),
-                               P.R * P.inv_cv * (1.f / 12.f), P.a * P.inv_cv * (1.f / 12.f)};
+                               P.R * P.inv_cv * (1.f / 12.f), P.a * P.inv_cv * (1.f / 12.f), ldexpf(1.f, -k)};
     for (int i = 0; i < KP_COUNT; ++i) P.kp[i] = make_float2(v[i], v[i]);
 }
 
