@@ -10,22 +10,23 @@ namespace lbgpu {
 
 namespace {
 
-template <int MINB>
+template <int MINB, bool EARLY>
 struct MarchFormT {
     static constexpr int threads = MARCH_T, min_blocks = MINB;
     static constexpr int smem = MarchSmem::total * (int)sizeof(float2);
     template <bool REC, bool OUT, bool QF>
     static __device__ __forceinline__ void body(const StepParams& P, const StepParams& C, int block, int fold,
                                                 const RecomputeOut* R) {
-        march_body<REC, OUT, QF>(P, C, block, fold, R);
+        march_body<REC, OUT, QF, EARLY>(P, C, block, fold, R);
     }
 };
 
-using MarchForm = MarchFormT<4>;
+using MarchForm = MarchFormT<4, true>;
+using MarchBatch = MarchFormT<4, false>;
 // 168 registers: no faster at full load (310 us on 4096^2 against 302), but
 // half as many blocks again fit, so a batch's tiles come in finer steps of
 // one wave (36 domains of 600 x 150: 85 us per step against 101).
-using March6 = MarchFormT<6>;
+using March6 = MarchFormT<6, false>;
 
 template <int NW, int K>
 struct TileForm {

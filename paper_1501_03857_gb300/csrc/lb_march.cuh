@@ -54,7 +54,13 @@ struct MarchSmem {
 // The whole step for block `block`: column pair block % npair, segment of
 // P.seg_h rows. C supplies the model constants (see lb_step_batch.cu); fold: the
 // previous step's q(t) is still to be folded.
-template <bool REC, bool OUT, bool QF>
+// EARLY: the next rows' loads between the collisions instead of after the
+// stores: a load does not overtake a store that it might alias, so it waits
+// where it stands. One domain: 4096^2 298 us instead of 306, 2048^2 86.4
+// instead of 88.4, 517 x 1003 24.6 instead of 24.8. Not for batches: 48 uneven
+// domains take 0.9 % longer with it, and in 168 registers it spills 200 bytes
+// more.
+template <bool REC, bool OUT, bool QF, bool EARLY>
 __device__ __forceinline__ void march_body(const StepParams& P, const StepParams& C, const int block, const int fold,
                                            const RecomputeOut* R) {
     extern __shared__ float2 sm2[];
@@ -216,25 +222,35 @@ __device__ __forceinline__ void march_body(const StepParams& P, const StepParams
             const Flow qa = flow(w0, w1, w2, fp, rhop, L - 1, 0);
             const Flow qb = flow(w1, w2, w3, f0, rho0, L, 1);
             vx0 = qa.vx, vy0 = qa.vy, vx1 = qb.vx, vy1 = qb.vy;
-            if (OUT) {
-                P2 wa[9], wb[9];
-                if (S || mine(L - 1)) {
-                    collide2(fp, qa.rho, qa.vx, qa.vy, qa.Fx, qa.Fy, qa.g2, C, wa);
-                    store(wa, qa.rho, L - 1);
-                }
-                if (S || mine(L)) {
-                    collide2(f0, qb.rho, qb.vx, qb.vy, qb.Fx, qb.Fy, qb.g2, C, wb);
-                    store(wb, qb.rho, L);
+            // the next two rows' loads, most of an iteration ahead
+            const bool more = S || L + 2 < ye + HALO;
+            auto shift = [&] {
+#pragma unroll
+                for (int a = 0; a < 9; ++a) fp[a] = f1[a];
+                rhop = rho1;
+            };
+            auto load0 = [&] { load_row2<S>(P, S ? L + 2 : phys(L + 2), c, f0, th0); };
+            auto load1 = [&] { load_row2<S>(P, S ? L + 3 : phys(L + 3), c, f1, th1); };
+            const bool sa = OUT && (S || mine(L - 1)), sb = OUT && (S || mine(L));
+            P2 wa[9], wb[9];
+            if (sa) {
+                collide2(fp, qa.rho, qa.vx, qa.vy, qa.Fx, qa.Fy, qa.g2, C, wa);
+                store(wa, qa.rho, L - 1);
+            }
+            if (EARLY) {
+                shift();
+                if (more) load1();
+            }
+            if (sb) collide2(f0, qb.rho, qb.vx, qb.vy, qb.Fx, qb.Fy, qb.g2, C, wb);
+            if (EARLY && more) load0();
+            if (sb) store(wb, qb.rho, L);
+            if (!EARLY) {
+                shift();
+                if (more) {
+                    load0();
+                    load1();
                 }
             }
-        }
-        // the next two rows' loads, a whole iteration minus P and B ahead
-#pragma unroll
-        for (int a = 0; a < 9; ++a) fp[a] = f1[a];
-        rhop = rho1;
-        if (S || L + 2 < ye + HALO) {
-            load_row2<S>(P, S ? L + 2 : phys(L + 2), c, f0, th0);
-            load_row2<S>(P, S ? L + 3 : phys(L + 3), c, f1, th1);
         }
         __syncthreads();
 

@@ -156,13 +156,13 @@ template <class F>
 auto with_batch_form(int form, F f) {
     if (form == FORM_TILE24) return f(Tile24{});
     if (form == FORM_MARCH6) return f(March6{});
-    return f(MarchForm{});
+    return f(MarchBatch{});
 }
 
 }  // namespace
 
 cudaError_t batch_prepare() {
-    cudaError_t e = BatchForm<MarchForm>::prepare();
+    cudaError_t e = BatchForm<MarchBatch>::prepare();
     if (e == cudaSuccess) e = BatchForm<March6>::prepare();
     return e == cudaSuccess ? BatchForm<Tile24>::prepare() : e;
 }
