@@ -167,8 +167,9 @@ int lb_mass(lb_handle* h, double* mass);
 /* Wait for the stream and report latched device faults. */
 int lb_sync(lb_handle* h);
 
-/* Number of steps taken, and the launch shape in use: threads per block and
- * rows per segment. */
+/* Number of steps taken, and the launch shape in use: block_x and seg_rows as
+ * lb_set_launch takes them (given back to it they choose the same shape), and
+ * the number of blocks. */
 int lb_info(lb_handle* h, int64_t* steps, int* block_x, int* seg_rows, int* nblocks);
 
 /* Override the launch shape of the fused step: block_x names its form (64:
@@ -305,8 +306,8 @@ int lb_batch_fields(lb_batch* b, int i, float* rho, float* ux, float* uy, float*
 int lb_batch_set_wall_temperature(lb_batch* b, int i, const double* Tb_profile, double superheat);
 int lb_batch_set_wettability(lb_batch* b, int i, double Gw);
 
-/* Steps taken, block size and blocks per launch (the persistent grid in
- * persistent mode). */
+/* Steps taken, block_x as lb_batch_set_launch takes it, and blocks per launch
+ * (the persistent grid in persistent mode). */
 int lb_batch_info(lb_batch* b, int64_t* steps, int* block_x, int* nblocks);
 
 /* Wait and report latched device faults of any instance: every instance's

@@ -341,7 +341,7 @@ int form_launch(int form, const lb_grid& g, int seg_rows, int nsm, Launch* out, 
     LB_CUDA(step_occupancy(form, &threads, occ), "occupancy");
     if (*occ < 1) return fail(LB_E_INVAL, "the fused step's block of %d threads does not fit on an SM", threads);
     out->form = form;
-    out->block_x = threads;
+    out->block_x = form_marches(form) ? 64 : form == FORM_TILE24 ? 128 : 256;
     out->nstrips = form_strips(form, g.Lx);
     int seg = seg_rows;
     if (seg <= 0) {
@@ -1044,7 +1044,7 @@ struct lb_batch {
     std::vector<int> h_off;      // [n + 1]: first block (tile) of each instance
     std::vector<StepParams> h_table;
     int block_x, seg_req;        // launch shape asked for (seg_req 0: automatic)
-    int form, threads;           // the form in use and its block size
+    int form;                    // the form in use
     int nblocks;
     bool dirty;                  // tables no longer match the instances' buffers
     int64_t steps;
@@ -1177,7 +1177,6 @@ int batch_layout(lb_batch* b) {
         if (form != FORM_MARCH && us >= best) continue;
         best = us;
         b->form = form;
-        b->threads = threads;
         occ = o;
         S = height;
     }
@@ -1186,7 +1185,7 @@ int batch_layout(lb_batch* b) {
         lb_handle* h = b->inst[i];
         const int nstrips = form_strips(b->form, h->grid.Lx);
         const int seg = b->seg_req > 0 ? b->seg_req : ceil_div(h->grid.Ly, ceil_div(h->grid.Ly, S));
-        h->launch = Launch{b->form, b->threads, seg, nstrips, ceil_div(h->grid.Ly, seg)};
+        h->launch = Launch{b->form, b->block_x, seg, nstrips, ceil_div(h->grid.Ly, seg)};
         apply_launch(h->base, h->launch);
         b->h_off[i + 1] = b->h_off[i] + nstrips * h->launch.nseg;
     }
@@ -1575,7 +1574,7 @@ int lb_batch_set_wettability(lb_batch* b, int i, double Gw) {
 int lb_batch_info(lb_batch* b, int64_t* steps, int* block_x, int* nblocks) {
     if (!b) return fail(LB_E_INVAL, "null batch");
     if (steps) *steps = b->steps;
-    if (block_x) *block_x = b->threads;
+    if (block_x) *block_x = b->block_x;
     if (nblocks) *nblocks = b->tpb > 0 ? b->pgrid : b->nblocks;
     return LB_OK;
 }

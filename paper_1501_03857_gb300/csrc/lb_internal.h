@@ -13,7 +13,8 @@ namespace lbgpu {
 enum Form { FORM_MARCH, FORM_TILE24, FORM_TILE16, FORM_TILE14, FORM_TILE12, FORM_COUNT, FORM_MARCH6 = FORM_COUNT };
 
 // Launch shape of the fused step: nstrips x nseg blocks of seg_rows rows
-// each; block_x threads per block (the form's).
+// each; block_x is the form's name to callers (lb_set_launch), with which and
+// seg_rows the same shape is chosen again.
 struct Launch {
     int form, block_x, seg_rows, nstrips, nseg;
 };
