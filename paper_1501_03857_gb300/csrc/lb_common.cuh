@@ -76,7 +76,7 @@ __device__ __forceinline__ void fold_heat(const StepParams& P, const int lane) {
     for (int x = lane; x < P.Lx; x += 512) {  // 16 loads in flight
         double v[16];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] = x + 32 * j < P.Lx ? __ldcg(P.qprev + x + 32 * j) : 0.0;
+        for (int j = 0; j < 16; ++j) v[j] = x + 32 * j < P.Lx ? lb_ldcg(P.qprev + x + 32 * j, P.qprev, P.Lx, P.acc) : 0.0;
 #pragma unroll
         for (int j = 0; j < 16; ++j) s[j & 3] += v[j];
     }

@@ -101,7 +101,8 @@ __device__ __forceinline__ bool finite_f(float v) { return fabsf(v) <= 3.4028234
 // runs (kernels overlap their predecessor, grid_start; the persistent batch's
 // blocks exchange buffers), are plain coherent ones (lb_ldco): after the wait
 // they see those writes, where the read-only path (lb_ldg, for the wall
-// temperature, which only copies write) may serve data it cached before.
+// temperature, which only copies write) may serve data it cached before; the
+// terms of q(t) are read at L2 (lb_ldcg).
 #ifdef LB_CHECKED
 __device__ __forceinline__ bool lb_inside(const void* p, const void* base, size_t bytes, size_t width, Acc* acc) {
     const char* c = static_cast<const char*>(p);
@@ -110,19 +111,31 @@ __device__ __forceinline__ bool lb_inside(const void* p, const void* base, size_
     atomicOr(&acc->err, ERR_BOUNDS);
     return false;
 }
-__device__ __forceinline__ float lb_ldg(const float* p, const float* base, size_t n, Acc* acc) {
-    return lb_inside(p, base, n * sizeof(float), sizeof(float), acc) ? __ldg(p) : 0.f;
+template <class T>
+__device__ __forceinline__ T lb_ldg(const T* p, const T* base, size_t n, Acc* acc) {
+    return lb_inside(p, base, n * sizeof(T), sizeof(T), acc) ? __ldg(p) : T(0);
 }
-__device__ __forceinline__ void lb_st(float* p, float v, const float* base, size_t n, Acc* acc) {
-    if (lb_inside(p, base, n * sizeof(float), sizeof(float), acc)) *p = v;
+template <class T>
+__device__ __forceinline__ void lb_st(T* p, T v, const T* base, size_t n, Acc* acc) {
+    if (lb_inside(p, base, n * sizeof(T), sizeof(T), acc)) *p = v;
 }
-__device__ __forceinline__ float lb_ldco(const float* p, const float* base, size_t n, Acc* acc) {
-    return lb_inside(p, base, n * sizeof(float), sizeof(float), acc) ? *p : 0.f;
+template <class T>
+__device__ __forceinline__ T lb_ldco(const T* p, const T* base, size_t n, Acc* acc) {
+    return lb_inside(p, base, n * sizeof(T), sizeof(T), acc) ? *p : T(0);
+}
+template <class T>
+__device__ __forceinline__ T lb_ldcg(const T* p, const T* base, size_t n, Acc* acc) {
+    return lb_inside(p, base, n * sizeof(T), sizeof(T), acc) ? __ldcg(p) : T(0);
 }
 #else
-__device__ __forceinline__ float lb_ldg(const float* p, const float*, size_t, Acc*) { return __ldg(p); }
-__device__ __forceinline__ float lb_ldco(const float* p, const float*, size_t, Acc*) { return *p; }
-__device__ __forceinline__ void lb_st(float* p, float v, const float*, size_t, Acc*) { *p = v; }
+template <class T>
+__device__ __forceinline__ T lb_ldg(const T* p, const T*, size_t, Acc*) { return __ldg(p); }
+template <class T>
+__device__ __forceinline__ void lb_st(T* p, T v, const T*, size_t, Acc*) { *p = v; }
+template <class T>
+__device__ __forceinline__ T lb_ldco(const T* p, const T*, size_t, Acc*) { return *p; }
+template <class T>
+__device__ __forceinline__ T lb_ldcg(const T* p, const T*, size_t, Acc*) { return __ldcg(p); }
 #endif
 // A store that only lanes with `on` make, as one predicated instruction: a
 // branch around a group of stores would end the basic block and with it the

@@ -166,8 +166,8 @@ __device__ __forceinline__ void march_body(const StepParams& P, const StepParams
         // ---- bottom-wall heat flux of level t (Sec. 3.2), one term per column
         if (QF && !S && !periodic && ys == 0 && L == 2) {
             const P2 r0 = own(bp + M::RHO + MW), a0 = own(t1), a1 = own(t1 + MW), a2 = own(t0);
-            if (outa) P.qpart[c.a] = heat_term(r0.x(), a0.x(), a1.x(), a2.x());
-            if (outb) P.qpart[c.b] = heat_term(r0.y(), a0.y(), a1.y(), a2.y());
+            if (outa) lb_st(P.qpart + c.a, heat_term(r0.x(), a0.x(), a1.x(), a2.x()), P.qpart, P.Lx, P.acc);
+            if (outb) lb_st(P.qpart + c.b, heat_term(r0.y(), a0.y(), a1.y(), a2.y()), P.qpart, P.Lx, P.acc);
         }
 
         // ---- B: rows L - 1, L

@@ -147,8 +147,8 @@ __device__ __forceinline__ void tile_rows(const StepParams& P, const StepParams&
         float2* q0 = at(sm + (HALO + 1) * TILE_ROW + 1 + lane);  // row y = 0
         const float2 rw = q0[RHO * Sh::field];
         const float2 t0 = q0[TH * Sh::field], t1 = q0[TH * Sh::field + TILE_ROW], t2 = q0[TH * Sh::field + 2 * TILE_ROW];
-        if (outa) P.qpart[c.a] = heat_term(rw.x, t0.x, t1.x, t2.x);
-        if (outb) P.qpart[c.b] = heat_term(rw.y, t0.y, t1.y, t2.y);
+        if (outa) lb_st(P.qpart + c.a, heat_term(rw.x, t0.x, t1.x, t2.x), P.qpart, P.Lx, P.acc);
+        if (outb) lb_st(P.qpart + c.b, heat_term(rw.y, t0.y, t1.y, t2.y), P.qpart, P.Lx, P.acc);
     }
 
     // ---- B: forces and velocity

@@ -75,3 +75,13 @@ def test_read_backs_run_on_their_own_device():
     assert seen == 4
     asked = [args for _, args in calls(text, "on_device_memory") if not args.startswith("const void*")]
     assert len(asked) == 4 and all(a.endswith("h->dev") for a in asked)
+
+
+def test_heat_flux_terms_go_through_the_checked_accesses():
+    """The checked build sees every global access of the step: the columns'
+    terms of q(t) too."""
+    for name in OVERLAPPED:
+        text = source(name)
+        assert not re.search(r"\bP\.q(part|prev)\s*\[", text), name
+        plain = [a for fn in ("__ldcg", "__ldg", "__stcg") for _, a in calls(text, fn) if "P.q" in a]
+        assert not plain, (name, plain)
