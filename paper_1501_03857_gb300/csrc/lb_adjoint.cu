@@ -947,9 +947,6 @@ cudaError_t adjoint_reverse_step(const ReverseShape& S, const StepParams& P, con
     A.u2 = R.u2;
     A.u3 = R.u3;
     A.u4 = R.u4;
-    // the four RK stages transposed, then the collision, forces, psi and the
-    // pull: two column-marching launches, segments sized so that the blocks
-    // fill the GPU once
     const int nsm = S.nsm, occ_t = S.occ_t, occ_f = S.occ_f;
     const int tiles = (P.Lx + RV_COLS - 1) / RV_COLS * rev_tiles<RevShape2<RV_NW, RV_K>>(P.Ly);
     // the tiles while they come to one wave (one block per SM, 13 us; a step of
@@ -962,10 +959,14 @@ cudaError_t adjoint_reverse_step(const ReverseShape& S, const StepParams& P, con
         Q.th_in = theta;
         return launch_after(rev_tile<RV_NW, RV_K>, tiles, RV_NW * 32, RV_SMEM, st, Q, A, lq);
     }
-    // (a floor of 4 rows per segment: on small domains more, shorter marches
-    // beat fewer long ones despite the halo rows; measured cost of the 256^2,
-    // 2000-step adjoint against its forward steps: 2.78x at 4, 2.90x at 1,
-    // 3.11x at 8, 4.06x at 16; at 512^2: 3.48x, 3.67x, 3.60x, 4.27x)
+    // (a floor of 4 rows per segment, which holds where the strips alone fill
+    // much of the GPU; a step of the whole adjoint, us, with a floor of 1, 4, 6,
+    // 8, 16 rows: 400 x 300 39.2, 36.3, 39.4, 38.7, 48.3; 2000 x 100 42.7, 41.4,
+    // 40.3, 43.3, 50.2; 1250 x 131 41.2, 40.6, 39.9, 42.7, 49.3; 8000 x 25 47.9,
+    // 47.3, 46.3, 47.2, 52.3)
+    // the four RK stages transposed, then the collision, forces, psi and the
+    // pull: two column-marching launches, segments sized so that the blocks
+    // fill the GPU once
     auto shape = [&](int nout, int occ, int& seg_h) {  // -> number of blocks
         const int nstrips = (P.Lx + nout - 1) / nout;
         const int nseg = std::max(1, nsm * occ / nstrips);

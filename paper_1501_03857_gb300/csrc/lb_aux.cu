@@ -7,6 +7,10 @@
 
 namespace lbgpu {
 
+// SMs of a GB300: caps the grids of kernels whose warps loop over the work
+// (any number of blocks gives the same result)
+constexpr int SMS = 152;
+
 namespace {
 
 __constant__ float kW[9] = {4.f / 9.f, 1.f / 9.f, 1.f / 9.f, 1.f / 9.f, 1.f / 9.f,
@@ -302,7 +306,7 @@ cudaError_t launch_copy_state(const float* f_src, float* f_dst, const float* t_s
     const int n0 = f_src ? 9 * Ly : 0, n1 = t_src ? Ly : 0;
     const uintptr_t all = (uintptr_t)f_src | (uintptr_t)f_dst | (uintptr_t)t_src | (uintptr_t)t_dst;
     const long long warps = (long long)(n0 + n1) * ((Lx + 1023) / 1024);
-    const int blocks = (int)std::min<long long>((warps + 7) / 8, 16 * 152);
+    const int blocks = (int)std::min<long long>((warps + 7) / 8, 16 * SMS);
     if (blocks == 0) return cudaSuccess;
     // (the pitch is a multiple of 32 floats: the other side's rows decide)
     auto kernel = all % 16 == 0 && Lx % 4 == 0 ? copy_rows<4> : copy_rows<1>;
@@ -334,7 +338,7 @@ cudaError_t launch_fields(const StepParams& P, float* rho, float* ux, float* uy,
 cudaError_t launch_mass(const StepParams& P, const float* f, cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(&P.acc->mass, 0, sizeof(double), st);
     if (e != cudaSuccess) return e;
-    mass_kernel<<<std::min(8 * 152, (9 * P.Ly + 7) / 8), 256, 0, st>>>(P, f);
+    mass_kernel<<<std::min(8 * SMS, (9 * P.Ly + 7) / 8), 256, 0, st>>>(P, f);
     return cudaGetLastError();
 }
 

@@ -23,9 +23,10 @@ struct MarchFormT {
 
 using MarchForm = MarchFormT<4, true>;
 using MarchBatch = MarchFormT<4, false>;
-// 168 registers: no faster at full load (310 us on 4096^2 against 302), but
-// half as many blocks again fit, so a batch's tiles come in finer steps of
-// one wave (36 domains of 600 x 150: 85 us per step against 101).
+// 168 registers: no faster at full load (310 us on 4096^2 against 302 with the
+// loads after the stores in both), but half as many blocks again fit, so a
+// batch's tiles come in finer steps of one wave (36 domains of 600 x 150: 85
+// us per step against 101).
 using March6 = MarchFormT<6, false>;
 
 template <int NW, int K>

@@ -19,11 +19,12 @@ template <int NW, int K>
 struct RevShape2 {
     static constexpr int rows = NW * K, out = rows - 2 * RV_HALO, edge = rows - RV_HALO;
     static constexpr int field = (rows + 2) * TILE_ROW, slots = 10 * field;
+    static_assert(edge - out + 1 >= 2 && rows - edge + 1 >= 2, "the top two rows share a tile");
 };
 
 // Tiles in y of a domain of Ly rows, and the rows [ys, ye) of tile i. The top
 // two rows always share a tile (the outflow top adds to what row Ly - 2
-// stored): a last tile of one row takes a second from its neighbour.
+// stored): with two tiles or more the last has at least edge - out + 1 rows.
 template <class Sh>
 __host__ __device__ __forceinline__ int rev_tiles(int Ly) {
     if (Ly <= Sh::rows) return 1;
@@ -35,8 +36,7 @@ __host__ __device__ __forceinline__ void rev_rows(int Ly, int i, int nt, int& ys
     auto start = [&](int k) {
         if (k == 0) return 0;
         if (k == nt) return Ly;
-        const int s = Sh::edge + (k - 1) * Sh::out;
-        return k == nt - 1 && Ly - s < 2 ? Ly - 2 : s;
+        return Sh::edge + (k - 1) * Sh::out;
     };
     ys = start(i);
     ye = start(i + 1);

@@ -2,7 +2,7 @@
 // temperature, wall heat flux, in one kernel. It has two forms with the same
 // arithmetic per cell (lb_cell.cuh) and so the same results bit for bit: a
 // marching one for domains that fill the GPU (lb_march.cuh) and a tiled one
-// for smaller ones (lb_tile.cuh, two tile heights); the host picks by the
+// for smaller ones (lb_tile.cuh, four tile heights); the host picks by the
 // measured times of each (compute_launch in lb_host.cu).
 #include "lb_forms.cuh"
 
