@@ -202,8 +202,10 @@ int lb_adjoint_scratch_bytes(lb_handle* h, int nsteps, int ckpt_every, size_t* b
 
 /* Checkpoint interval for lb_adjoint over nsteps steps whose scratch fits in
  * budget_bytes of device memory. 1 (every step's state and intermediates
- * stored, no replay: the fastest) when its scratch fits; otherwise the
- * interval with the smallest scratch (checkpoints take ~10 nsteps / C
+ * stored, no replay: the fastest on domains larger than L2; on smaller ones
+ * segments whose replay stays in L2 can be faster, by a sixth on 256 x 256 with
+ * 100 steps a segment) when its scratch fits; otherwise the interval with the
+ * smallest scratch (checkpoints take ~10 nsteps / C
  * planes and the replay buffers ~40 C, so about C = sqrt(nsteps / 4)), whose
  * run time is about the same for every C >= 2 (each step is replayed once).
  * Writes the interval to *ckpt_every and, if bytes is not NULL, its scratch

@@ -23,13 +23,14 @@
 // registers (carried from the iteration that made them), the RK coefficients
 // of a row once for the two stages that follow each other on it.
 //
-// What bounds it: eight warps per SM (254 registers) keep the FP32 pipe 53 %
-// and the shared-memory path 53 % busy, with fixed-latency waits as the first
+// What bounds it: eight warps per SM (240 registers) keep the FP32 pipe 54 %
+// and the shared-memory path 54 % busy, with fixed-latency waits as the first
 // stall; twelve warps (168 registers) measure the same. On 4096^2: one row
 // per iteration 351 us; two rows 325 us; square root and stores without
 // branches, so that the two rows interleave, 320 us; own values from
-// registers, 302 us (369 instructions per cell instead of 541, shared-load
-// wavefronts 53 instead of 110 per cell-warp).
+// registers, 302 us (392 instructions per cell instead of 541, shared-load
+// wavefronts 56 instead of 110 per cell-warp); coherent loads 306 us, between
+// the collisions 298 us.
 #pragma once
 
 #include "lb_common.cuh"

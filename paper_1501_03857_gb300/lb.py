@@ -371,8 +371,8 @@ class Simulation:
         """J = mean wall heat flux over the next nsteps steps and its gradients
         dJ/d(T_b(x) - T_s) [Lx] and dJ/dG_w by the discrete adjoint
         (lb_adjoint), with a checkpoint every ckpt_every steps; ckpt_every = 1
-        stores every step and replays none (faster, about 20 planes of
-        scratch per step); None picks it with adjoint_ckpt (every step stored
+        stores every step and replays none (faster on domains larger than
+        L2; about 20 planes of scratch per step); None picks it with adjoint_ckpt (every step stored
         whenever that takes at most half the free device memory). Advances
         the simulation by nsteps."""
         torch = self.torch
